@@ -16,6 +16,7 @@
 #include "pt_bin.h"
 #include "pt_ctx.h"
 #include "pt_internal.h"
+#include "pt_map.cuh"
 
 namespace pt {
 int fam_g2_fp64_push(int, const PushArgs&, int, int, void*);
@@ -333,6 +334,90 @@ static T* dmalloc(pt_ctx* c, size_t n, cudaError_t* err) {
   return (T*)p;
 }
 
+// Monomial coefficients of the element map (pt_map.cuh), one thread per
+// element and coordinate: the nodal values taken to powers of xi1, xi2, xi3 in
+// turn by V (V[k g + a]: the xi^k coefficient of the Lagrange basis l_a on the
+// equidistant nodes), in FP64, then split in two FP32 parts.
+struct MonoBasis {
+  double v[PT_MAXG * PT_MAXG];
+};
+
+template <int G>
+__global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tmask, int nelem,
+                       const MonoBasis V, float* __restrict__ hi, float* __restrict__ lo) {
+  constexpr int G3 = G * G * G, AP = Mono<G>::AP, CS = Mono<G>::CS;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 3 * nelem) return;
+  const int e = i / 3, r = i - 3 * e;
+  const double* X = xg + (size_t)e * 3 * G3 + r;
+  float* h = hi + (size_t)i * CS;
+  float* l = lo + (size_t)i * CS;
+  auto put = [&](int q, double v) {
+    h[q] = (float)v;
+    l[q] = (float)(v - (double)h[q]);
+  };
+  if ((tmask[e] >> r) & 1) {  // 8 coefficients of the corner interpolant
+    for (int q = 0; q < 8; ++q) {
+      double v = 0.0;
+      for (int w = 0; w < 8; ++w) {
+        const double xv = X[3 * (((w & 1) ? G - 1 : 0) +
+                                 G * (((w & 2) ? G - 1 : 0) + G * ((w & 4) ? G - 1 : 0)))];
+        v += (__popc(q & ~w) & 1) ? -xv : xv;
+      }
+      put(q, 0.125 * v);
+    }
+    for (int q = 8; q < CS; ++q) h[q] = l[q] = 0.f;
+    return;
+  }
+  double T[G3];
+  for (int q = 0; q < G3; ++q) T[q] = X[3 * q];
+  for (int st = 1; st < G3; st *= G)
+    for (int q = 0; q < G3; ++q) {
+      if ((q / st) % G) continue;
+      double w[G];
+      for (int a = 0; a < G; ++a) w[a] = T[q + a * st];
+      for (int kk = 0; kk < G; ++kk) {
+        double v = 0.0;
+        for (int a = 0; a < G; ++a) v += V.v[kk * G + a] * w[a];
+        T[q + kk * st] = v;
+      }
+    }
+  for (int q = 0; q < CS; ++q) h[q] = l[q] = 0.f;
+  for (int c = 0; c < G; ++c)
+    for (int b = 0; b < G; ++b)
+      for (int a = 0; a < G; ++a) put(AP * (c + G * b) + a, T[a + G * (b + G * c)]);
+}
+
+static int mono_floats(int g) {
+  return g == 2 ? Mono<2>::CS : g == 3 ? Mono<3>::CS : g == 4 ? Mono<4>::CS : Mono<5>::CS;
+}
+
+static cudaError_t launch_mono(pt_ctx* c) {
+  MonoBasis V;
+  for (int a = 0; a < c->g; ++a) {
+    // coefficients of prod_{m != a} (x - x_m) / (x_a - x_m)
+    double p[PT_MAXG] = {1.0, 0.0, 0.0, 0.0, 0.0};
+    int deg = 0;
+    const double xa = -1.0 + 2.0 * a / (c->g - 1);
+    for (int m = 0; m < c->g; ++m) {
+      if (m == a) continue;
+      const double xm = -1.0 + 2.0 * m / (c->g - 1), s = 1.0 / (xa - xm);
+      for (int q = ++deg; q >= 0; --q)
+        p[q] = s * ((q > 0 ? p[q - 1] : 0.0) - (q < deg ? xm * p[q] : 0.0));
+    }
+    for (int q = 0; q < c->g; ++q) V.v[q * c->g + a] = p[q];
+  }
+  const int nb = (3 * c->nelem + 127) / 128;
+  switch (c->g) {
+    case 2: k_mono<2><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
+    case 3: k_mono<3><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
+    case 4: k_mono<4><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
+    default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
+  }
+  const cudaError_t err = cudaGetLastError();
+  return err ? err : cudaStreamSynchronize(c->stream);
+}
+
 static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
   const int E = md->nelem, g = md->ngeo + 1, g3 = g * g * g;
   c->nelem = E;
@@ -340,7 +425,7 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
   c->g = g;
   std::vector<double> xg64((size_t)E * g3 * 3), ce((size_t)E * 3), bil((size_t)E * 72),
       shift((size_t)E * 18);
-  std::vector<float> xg32((size_t)E * g3 * 3), xg32lo((size_t)E * g3 * 3), tri((size_t)E * 12), slab((size_t)E * 48, 0.f);
+  std::vector<float> xg32((size_t)E * g3 * 3), tri((size_t)E * 12), slab((size_t)E * 48, 0.f);
   std::vector<int> fnbr((size_t)E * 6), finfo((size_t)E * 6), tmask((size_t)E, 0);
   std::vector<double> M;
   bezier_matrix(g, M);
@@ -365,9 +450,7 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
       for (int r = 0; r < 3; ++r) {
         double v = X[3 * q + r] - cc[r];
         xg64[((size_t)e * g3 + q) * 3 + r] = v;
-        const float vh = (float)v;
-        xg32[(size_t)e * 3 * g3 + r * g3 + q] = vh;
-        xg32lo[(size_t)e * 3 * g3 + r * g3 + q] = (float)(v - (double)vh);
+        xg32[(size_t)e * 3 * g3 + r * g3 + q] = (float)v;
         Rmax = std::max(Rmax, std::fabs(v));
       }
     for (int r = 0; r < 3; ++r) ce[3 * e + r] = cc[r];
@@ -561,7 +644,10 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_xg32 = dmalloc<float>(cc, xg32.size(), &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
-  c->d_xg32lo = dmalloc<float>(cc, xg32lo.size(), &err);
+  const size_t nmono = (size_t)E * 3 * mono_floats(g);
+  c->d_mono = dmalloc<float>(cc, nmono, &err);
+  if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
+  c->d_monolo = dmalloc<float>(cc, nmono, &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_ce = dmalloc<double>(cc, ce.size(), &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
@@ -593,7 +679,6 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
     const void* h;
     size_t b;
   } cp[] = {{c->d_xg64, xg64.data(), xg64.size() * 8}, {c->d_xg32, xg32.data(), xg32.size() * 4},
-            {c->d_xg32lo, xg32lo.data(), xg32lo.size() * 4},
             {c->d_ce, ce.data(), ce.size() * 8},       {c->d_tri, tri.data(), tri.size() * 4},
             {c->d_tmask, tmask.data(), tmask.size() * 4},
             {c->d_fnbr, fnbr.data(), fnbr.size() * 4}, {c->d_finfo, finfo.data(), finfo.size() * 4},
@@ -605,6 +690,8 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
     err = cudaMemcpy(q.d, q.h, q.b, cudaMemcpyHostToDevice);
     if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMemcpy: %s", cudaGetErrorString(err));
   }
+  err = launch_mono(c);
+  if (err) return fail(nullptr, PT_ERR_CUDA, "element map: %s", cudaGetErrorString(err));
   return PT_OK;
 }
 
@@ -623,10 +710,6 @@ static void fill_consts(const pt_ctx* c, DevConsts& k) {
     k.gw[a] = gw[a];
     k.gn32[a] = (float)gn[a];
     k.gw32[a] = (float)gw[a];
-    k.gn_hi[a] = (float)gn[a];
-    k.gn_lo[a] = (float)(gn[a] - (double)k.gn_hi[a]);
-    k.gw_hi[a] = (float)gw[a];
-    k.gw_lo[a] = (float)(gw[a] - (double)k.gw_hi[a]);
   }
   for (int i = 0; i < c->N + 1 && c->N >= 0; ++i) {
     k.sn[i] = c->sn[i];
@@ -675,7 +758,8 @@ static DevMesh dev_mesh(const pt_ctx* c) {
   m.g = c->g;
   m.xg64 = c->d_xg64;
   m.xg32 = c->d_xg32;
-  m.xg32lo = c->d_xg32lo;
+  m.mono = c->d_mono;
+  m.monolo = c->d_monolo;
   m.ce = c->d_ce;
   m.tri = c->d_tri;
   m.tmask = c->d_tmask;
@@ -948,7 +1032,7 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   else bytes += 2 * al(12 * nn);                      // xh, xl
   bytes += 3 * al(3 * rs * nn) + al(rs * nn);         // v, kx, kv, d
   bytes += al((f64 ? 24 : 24) * nn);                  // xe
-  bytes += f64 ? 0 : al(12 * nn) + 2 * al(12 * nn);   // guess, converged xi (hi, lo)
+  bytes += f64 ? 0 : al(12 * nn);                     // guess
   bytes += 4 * al(4 * nn) + 256;                      // e, hits, st, list, counters
   if (c->state_cap < n || !c->d_state) {
     if (c->d_state) cudaFree(c->d_state);
@@ -966,7 +1050,6 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   a.x = nullptr;
   a.xh = a.xl = nullptr;
   a.guess = nullptr;
-  a.xih = a.xil = nullptr;
   if (f64) {
     a.x = (double*)take(24 * nn);
   } else {
@@ -980,8 +1063,6 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   a.xe = take(24 * nn);
   if (!f64) {
     a.guess = (float*)take(12 * nn);
-    a.xih = (float*)take(12 * nn);
-    a.xil = (float*)take(12 * nn);
   }
   a.e = (int*)take(4 * nn);
   a.hits = (int*)take(4 * nn);

@@ -21,7 +21,8 @@ struct pt_ctx {
   int nelem = 0, ngeo = 0, g = 0, ncurved = 0;
   double* d_xg64 = nullptr;
   float* d_xg32 = nullptr;
-  float* d_xg32lo = nullptr;
+  float* d_mono = nullptr;
+  float* d_monolo = nullptr;
   double* d_ce = nullptr;
   float* d_tri = nullptr;
   int* d_tmask = nullptr;

@@ -12,23 +12,8 @@
 
 #include "pt_df.cuh"
 #include "pt_internal.h"
+#include "pt_map.cuh"
 
-// 1: evaluate the per-dimension Lagrange bases of the Newton residuals in a
-// rolled loop (one copy of the code, values through local memory), which
-// shrinks the hot loop's instruction footprint
-#ifndef PT_ROLL_BASIS
-#define PT_ROLL_BASIS 1
-#endif
-// 1: run-time indices into small register arrays of the interpolation
-// (PT_PICK_INTERP) and of the element map (PT_PICK_MAP) go through chains of
-// selects instead of dynamic indexing, which keeps the arrays out of local
-// memory at the cost of more live registers
-#ifndef PT_PICK_INTERP
-#define PT_PICK_INTERP 0
-#endif
-#ifndef PT_PICK_MAP
-#define PT_PICK_MAP 0
-#endif
 // FP32 Newton iterations of the FP32 mode stop once the step is below this;
 // the final iterations (double-float residuals, last FP32 inverse Jacobian)
 // take over and converge linearly with a factor of about the step at which
@@ -56,25 +41,6 @@ __device__ __forceinline__ T tabs(T a) {
 template <typename T>
 __device__ __forceinline__ T tmax3(T a, T b, T c) {
   return fmax(fmax(tabs(a), tabs(b)), tabs(c));
-}
-
-// a[i] for a run-time i without indexing the array dynamically (which would
-// put it in local memory): a chain of selects over the unrolled indices
-template <int N, typename T>
-__device__ __forceinline__ T pick(const T* a, int i) {
-  T v = a[0];
-#pragma unroll
-  for (int j = 1; j < N; ++j)
-    if (j == i) v = a[j];
-  return v;
-}
-
-// a[i] = v for a run-time i, likewise
-template <int N, typename T>
-__device__ __forceinline__ void put(T* a, int i, T v) {
-#pragma unroll
-  for (int j = 0; j < N; ++j)
-    if (j == i) a[j] = v;
 }
 
 template <typename T>
@@ -152,40 +118,6 @@ __device__ __forceinline__ void lagr_d(T x, const T* nodes, const T* w, T* l, T*
   }
 }
 
-// Read-only load: through the non-coherent path from global memory, or (SH)
-// a generic load, for data that may sit in shared memory.
-template <bool SH, typename V>
-__device__ __forceinline__ V ldx(const V* p) {
-  if constexpr (SH)
-    return *p;
-  else
-    return __ldg(p);
-}
-
-// G consecutive floats starting at p (p is 16-byte aligned when G == 4 and
-// 8-byte aligned when G is even: row starts are multiples of G in arrays whose
-// per-element blocks are multiples of 16 bytes)
-template <int G, bool SH = false>
-__device__ __forceinline__ void load_row(const float* __restrict__ p, float* v) {
-  if constexpr (G == 4) {
-    const float4 q = ldx<SH>(reinterpret_cast<const float4*>(p));
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = q.z;
-    v[3] = q.w;
-  } else if constexpr (G % 2 == 0) {
-#pragma unroll
-    for (int i = 0; i < G; i += 2) {
-      const float2 q = ldx<SH>(reinterpret_cast<const float2*>(p + i));
-      v[i] = q.x;
-      v[i + 1] = q.y;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < G; ++i) v[i] = ldx<SH>(p + i);
-  }
-}
-
 template <typename T>
 __device__ __forceinline__ bool inv3(const T* J, T* Ji) {
   T c00 = J[4] * J[8] - J[5] * J[7];
@@ -213,142 +145,9 @@ __device__ __forceinline__ void matvec3(const T* M, const T* v, T* o) {
 }
 
 // ---------------------------------------------------------------------------
-// element map chi(xi) = sum_abc X_abc l_a(xi1) l_b(xi2) l_c(xi3), sum-factorised
+// element map chi(xi) = sum_abc X_abc l_a(xi1) l_b(xi2) l_c(xi3) and its inverse
+// (FP32 evaluation: pt_map.cuh)
 // ---------------------------------------------------------------------------
-
-// FP32, nodes coordinate-major [3][G^3]; chi and Jacobian J[r][q] = d chi_r / d xi_q
-template <int G>
-__device__ __forceinline__ int corner_node(int q) {
-  return ((q & 1) ? G - 1 : 0) + G * (((q & 2) ? G - 1 : 0) + G * ((q & 4) ? G - 1 : 0));
-}
-
-// FP32, nodes coordinate-major [3][G^3]; chi and Jacobian J[r][q] = d chi_r / d xi_q.
-// Coordinates flagged in tm are trilinear in xi: their 8-corner form is used.
-// Per-thread scratch for the per-dimension bases: SS = 0 keeps them in a
-// local array (computed in a rolled loop, read through local memory); SS > 0
-// puts them in shared memory at sb[row * SS] (sb: this thread's column of a
-// [rows][SS] block array), which keeps local memory out of the L1 cache.
-// With a shared-memory scratch (SS > 0), the small per-thread results that
-// the rolled loops index at run time (chi, J, a residual, the interpolation's
-// third-direction basis and its outputs) also go through rows of the scratch
-// from kScratchOut on instead of through local memory (PT_SMEM_OUT = 1).
-#ifndef PT_SMEM_OUT
-#define PT_SMEM_OUT 1
-#endif
-constexpr int kScratchOut = 6 * PT_MAXG;
-constexpr int kScratchRows = kScratchOut + 12;
-
-template <int SS>
-struct BasisStore {
-  float* sb;
-  float loc[SS > 0 ? 1 : 6 * PT_MAXG];
-  __device__ __forceinline__ float* row(int r) { return SS > 0 ? sb + r * SS : loc + r; }
-  __device__ __forceinline__ float get(int r) const { return SS > 0 ? sb[r * SS] : loc[r]; }
-};
-
-template <int G, int SS = 0, bool SH = false>
-__device__ __forceinline__ void map_j32(const float* __restrict__ X, const float* xi, int tm,
-                                        const DevConsts& k, float* chi, float* J,
-                                        float* sb = nullptr) {
-  constexpr int G3 = G * G * G;
-  // rows d G + i: l_i(xi_d); rows (3 + d) G + i: l_i'(xi_d)
-  BasisStore<SS> bs;
-  bs.sb = sb;
-  if (tm != 7) {
-#if PT_ROLL_BASIS
-#pragma unroll 1
-#else
-#pragma unroll
-#endif
-    for (int d = 0; d < 3; ++d) {
-      float l[G], dl[G];
-      lagr_d<G, float>(xi[d], k.gn32, k.gw32, l, dl);
-#pragma unroll
-      for (int i = 0; i < G; ++i) {
-        *bs.row(d * G + i) = l[i];
-        *bs.row((3 + d) * G + i) = dl[i];
-      }
-    }
-  }
-#define PT_L(d, i) bs.get((d) * G + (i))
-#define PT_D(d, i) bs.get((3 + (d)) * G + (i))
-  const float hp[3] = {0.5f * (1.f + xi[0]), 0.5f * (1.f + xi[1]), 0.5f * (1.f + xi[2])};
-  const float hm[3] = {0.5f * (1.f - xi[0]), 0.5f * (1.f - xi[1]), 0.5f * (1.f - xi[2])};
-  // one coordinate at a time; the loops over c and r stay rolled so that the
-  // hot loop's code stays small
-#pragma unroll 1
-  for (int r = 0; r < 3; ++r) {
-    const float* Xr = X + r * G3;
-    float cr = 0.f, j0 = 0.f, j1 = 0.f, j2 = 0.f;
-    if ((tm >> r) & 1) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float xv = ldx<SH>(Xr + corner_node<G>(q));
-        const float a0 = (q & 1) ? hp[0] : hm[0], a1 = (q & 2) ? hp[1] : hm[1],
-                    a2 = (q & 4) ? hp[2] : hm[2];
-        const float s0 = (q & 1) ? 0.5f : -0.5f, s1 = (q & 2) ? 0.5f : -0.5f,
-                    s2 = (q & 4) ? 0.5f : -0.5f;
-        cr = fmaf(xv, a0 * a1 * a2, cr);
-        j0 = fmaf(xv, s0 * a1 * a2, j0);
-        j1 = fmaf(xv, a0 * s1 * a2, j1);
-        j2 = fmaf(xv, a0 * a1 * s2, j2);
-      }
-    } else {
-#pragma unroll 1
-      for (int c = 0; c < G; ++c) {
-        float T0 = 0.f, T1 = 0.f, T2 = 0.f;
-#pragma unroll
-        for (int b = 0; b < G; ++b) {
-          float sv = 0.f, s1 = 0.f, row[G];
-          load_row<G, SH>(Xr + G * (b + G * c), row);
-#pragma unroll
-          for (int a = 0; a < G; ++a) {
-            sv = fmaf(row[a], PT_L(0, a), sv);
-            s1 = fmaf(row[a], PT_D(0, a), s1);
-          }
-          T0 = fmaf(sv, PT_L(1, b), T0);
-          T1 = fmaf(s1, PT_L(1, b), T1);
-          T2 = fmaf(sv, PT_D(1, b), T2);
-        }
-        const float lc = PT_L(2, c), dc = PT_D(2, c);
-        cr = fmaf(T0, lc, cr);
-        j0 = fmaf(T1, lc, j0);
-        j1 = fmaf(T2, lc, j1);
-        j2 = fmaf(T0, dc, j2);
-      }
-    }
-#if PT_PICK_MAP
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      if (q == r) {
-        chi[q] = cr;
-        J[3 * q] = j0;
-        J[3 * q + 1] = j1;
-        J[3 * q + 2] = j2;
-      }
-#else
-    if constexpr (SS > 0 && PT_SMEM_OUT) {
-      sb[(kScratchOut + r) * SS] = cr;
-      sb[(kScratchOut + 3 + 3 * r) * SS] = j0;
-      sb[(kScratchOut + 4 + 3 * r) * SS] = j1;
-      sb[(kScratchOut + 5 + 3 * r) * SS] = j2;
-    } else {
-      chi[r] = cr;
-      J[3 * r] = j0;
-      J[3 * r + 1] = j1;
-      J[3 * r + 2] = j2;
-    }
-#endif
-  }
-  if constexpr (SS > 0 && PT_SMEM_OUT && !PT_PICK_MAP) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) chi[q] = sb[(kScratchOut + q) * SS];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) J[q] = sb[(kScratchOut + 3 + q) * SS];
-  }
-}
-#undef PT_L
-#undef PT_D
 
 // FP64, nodes point-major [G^3][3]; with WJ also the Jacobian
 template <int G, bool WJ>
@@ -438,241 +237,6 @@ __device__ __forceinline__ bool newton64(const double* X64, const double* xl, do
   return false;
 }
 
-// Lagrange basis on the geometry nodes in double-float (nodes and barycentric
-// weights carried as hi + lo pairs)
-template <int NP>
-__device__ __forceinline__ void lagr_df(df x, const DevConsts& k, df* l) {
-  df d[NP];
-#pragma unroll
-  for (int m = 0; m < NP; ++m) d[m] = df_sub(x, df{k.gn_hi[m], k.gn_lo[m]});
-  df pre = df_from(1.f);
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    l[i] = pre;
-    if (i + 1 < NP) pre = df_mul(pre, d[i]);
-  }
-  df suf = df_from(1.f);
-#pragma unroll
-  for (int i = NP - 1; i >= 0; --i) {
-    l[i] = df_mul(df_mul(l[i], suf), df{k.gw_hi[i], k.gw_lo[i]});
-    if (i > 0) suf = df_mul(suf, d[i]);
-  }
-}
-
-// Residual chi(xi) - x of the element map in double-float, sum-factorised;
-// nodes as hi [3][G^3] + lo [3][G^3] (relative to the element centre);
-// coordinates flagged in tm use the 8-corner trilinear form.
-template <int G, int SS = 0, bool SH = false>
-__device__ __forceinline__ void resid_df(const float* __restrict__ Xh,
-                                         const float* __restrict__ Xl, const df* xi, int tm,
-                                         const df* xloc, const DevConsts& k, float* r,
-                                         float* sb = nullptr) {
-  constexpr int G3 = G * G * G;
-  // rows d G + i: high part of l_i(xi_d); rows (3 + d) G + i: low part
-  BasisStore<SS> bs;
-  bs.sb = sb;
-  if (tm != 7) {
-#if PT_ROLL_BASIS
-#pragma unroll 1
-#else
-#pragma unroll
-#endif
-    for (int d = 0; d < 3; ++d) {
-      df l[G];
-      lagr_df<G>(xi[d], k, l);
-#pragma unroll
-      for (int i = 0; i < G; ++i) {
-        *bs.row(d * G + i) = l[i].hi;
-        *bs.row((3 + d) * G + i) = l[i].lo;
-      }
-    }
-  }
-#define PT_LDF(d, i) df{bs.get((d) * G + (i)), bs.get((3 + (d)) * G + (i))}
-  df w8[8];
-  if (tm != 0) {
-    df hp[3], hm[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const df up = df_add(df_from(1.f), xi[d]);
-      const df dn = df_sub(df_from(1.f), xi[d]);
-      hp[d] = df{0.5f * up.hi, 0.5f * up.lo};
-      hm[d] = df{0.5f * dn.hi, 0.5f * dn.lo};
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const df w01 = df_mul((q & 1) ? hp[0] : hm[0], (q & 2) ? hp[1] : hm[1]);
-      w8[q] = df_mul(w01, hm[2]);
-      w8[q + 4] = df_mul(w01, hp[2]);
-    }
-  }
-#pragma unroll 1
-  for (int q = 0; q < 3; ++q) {
-    const float* Ph = Xh + q * G3;
-    const float* Pl = Xl + q * G3;
-    df_acc a3;
-    dacc_init(a3);
-    if ((tm >> q) & 1) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int i = corner_node<G>(c);
-        dacc_fma(a3, df{ldx<SH>(Ph + i), ldx<SH>(Pl + i)}, w8[c]);
-      }
-    } else {
-#pragma unroll 1
-      for (int c = 0; c < G; ++c) {
-        df_acc a2;
-        dacc_init(a2);
-#pragma unroll
-        for (int b = 0; b < G; ++b) {
-          df_acc a1;
-          dacc_init(a1);
-          float rh[G], rl[G];
-          load_row<G, SH>(Ph + G * (b + G * c), rh);
-          load_row<G, SH>(Pl + G * (b + G * c), rl);
-#pragma unroll
-          for (int a = 0; a < G; ++a) dacc_fma(a1, df{rh[a], rl[a]}, PT_LDF(0, a));
-          dacc_fma(a2, dacc_result(a1), PT_LDF(1, b));
-        }
-        dacc_fma(a3, dacc_result(a2), PT_LDF(2, c));
-      }
-    }
-#if PT_PICK_MAP
-    const df rr = df_sub(dacc_result(a3), pick<3>(xloc, q));
-    put<3>(r, q, __fadd_rn(rr.hi, rr.lo));
-#else
-    const df rr = df_sub(dacc_result(a3), xloc[q]);
-    if constexpr (SS > 0 && PT_SMEM_OUT)
-      sb[(kScratchOut + q) * SS] = __fadd_rn(rr.hi, rr.lo);
-    else
-      r[q] = __fadd_rn(rr.hi, rr.lo);
-#endif
-  }
-  if constexpr (SS > 0 && PT_SMEM_OUT && !PT_PICK_MAP) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) r[q] = sb[(kScratchOut + q) * SS];
-  }
-#undef PT_LDF
-}
-
-// Lagrange basis at z (l) and its increment dl = l(z + dz) - l(z), the latter
-// without cancellation: with f_m = z - x_m and F_m = f_m + dz, the product
-// difference telescopes, prod F - prod f = dz sum_j (prod_{i<j} f_i)(prod_{i>j} F_i),
-// so dl carries the relative accuracy of FP32 however small dz is.
-template <int G>
-__device__ __forceinline__ void lagr_inc(float z, float dz, const float* xn, const float* w,
-                                         float* l, float* dl) {
-  float f[G], F[G];
-#pragma unroll
-  for (int m = 0; m < G; ++m) {
-    f[m] = z - xn[m];
-    F[m] = f[m] + dz;
-  }
-#pragma unroll
-  for (int a = 0; a < G; ++a) {
-    float suf[G], sp = 1.f;
-#pragma unroll
-    for (int m = G - 1; m >= 0; --m) {
-      suf[m] = sp;
-      if (m != a) sp *= F[m];
-    }
-    float pre = 1.f, acc = 0.f;
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-      if (m == a) continue;
-      acc = fmaf(pre, suf[m], acc);
-      pre *= f[m];
-    }
-    l[a] = w[a] * pre;
-    dl[a] = w[a] * dz * acc;
-  }
-}
-
-// Increment of the element map between two nearby points, dchi = chi(z + dz) -
-// chi(z), in FP32 without cancellation: with L = l + dl the bases at z + dz,
-//   prod L - prod l = dl0 L1 L2 + l0 dl1 L2 + l0 l1 dl2
-// (and likewise for the 8-corner form of trilinear coordinates), so every term
-// carries a factor dl and the result has FP32 relative accuracy.  Used for the
-// second residual of the final Newton iterations: r(z + dz) = r(z) + dchi, with
-// r(z) from the double-float residual.  Nodes: FP32 high parts, relative to the
-// element centre (the low parts change dchi by ~1e-8 of itself).
-template <int G, bool SH = false, int SS = 0>
-__device__ __forceinline__ void map_inc32(const float* __restrict__ X, const float* z,
-                                          const float* dz, int tm, const DevConsts& k,
-                                          float* dchi, float* sb = nullptr) {
-  constexpr int G3 = G * G * G;
-  float l0[G], dl0[G], l1[G], dl1[G], l2[G], dl2[G];
-  lagr_inc<G>(z[0], dz[0], k.gn32, k.gw32, l0, dl0);
-  lagr_inc<G>(z[1], dz[1], k.gn32, k.gw32, l1, dl1);
-  lagr_inc<G>(z[2], dz[2], k.gn32, k.gw32, l2, dl2);
-  float hp[3], hm[3], dh[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    hp[d] = 0.5f * (1.f + z[d]);
-    hm[d] = 0.5f * (1.f - z[d]);
-    dh[d] = 0.5f * dz[d];
-  }
-#pragma unroll 1
-  for (int q = 0; q < 3; ++q) {
-    const float* Xq = X + q * G3;
-    float acc = 0.f;
-    if ((tm >> q) & 1) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const float a0 = (c & 1) ? hp[0] : hm[0], a1 = (c & 2) ? hp[1] : hm[1],
-                    a2 = (c & 4) ? hp[2] : hm[2];
-        const float d0 = (c & 1) ? dh[0] : -dh[0], d1 = (c & 2) ? dh[1] : -dh[1],
-                    d2 = (c & 4) ? dh[2] : -dh[2];
-        const float A1 = a1 + d1, A2 = a2 + d2;
-        const float dw = d0 * A1 * A2 + a0 * d1 * A2 + a0 * a1 * d2;
-        acc = fmaf(ldx<SH>(Xq + corner_node<G>(c)), dw, acc);
-      }
-    } else {
-      float t1 = 0.f, t2 = 0.f, t3 = 0.f;
-#pragma unroll 1
-      for (int c = 0; c < G; ++c) {
-        float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-        for (int b = 0; b < G; ++b) {
-          float row[G];
-          load_row<G, SH>(Xq + G * (b + G * c), row);
-          float A = 0.f, B = 0.f;
-#pragma unroll
-          for (int a = 0; a < G; ++a) {
-            A = fmaf(row[a], dl0[a], A);
-            B = fmaf(row[a], l0[a], B);
-          }
-          s1 = fmaf(A, l1[b] + dl1[b], s1);
-          s2 = fmaf(B, dl1[b], s2);
-          s3 = fmaf(B, l1[b], s3);
-        }
-        float lc = l2[0], dc = dl2[0];
-#pragma unroll
-        for (int j = 1; j < G; ++j)
-          if (j == c) {
-            lc = l2[j];
-            dc = dl2[j];
-          }
-        t1 = fmaf(s1, lc + dc, t1);
-        t2 = fmaf(s2, lc + dc, t2);
-        t3 = fmaf(s3, dc, t3);
-      }
-      acc = t1 + t2 + t3;
-    }
-#if PT_PICK_MAP
-    put<3>(dchi, q, acc);
-#else
-    if constexpr (SS > 0 && PT_SMEM_OUT)
-      sb[(kScratchOut + q) * SS] = acc;
-    else
-      dchi[q] = acc;
-#endif
-  }
-  if constexpr (SS > 0 && PT_SMEM_OUT && !PT_PICK_MAP) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) dchi[q] = sb[(kScratchOut + q) * SS];
-  }
-}
-
 template <int G>
 __device__ __noinline__ bool newton64_cold(const double* X64, const double* xl, double* xi,
                                            const DevConsts& k, int& it64) {
@@ -684,24 +248,20 @@ __device__ __noinline__ bool newton64_cold(const double* X64, const double* xl, 
 // 1e-5, then double-float residuals with the last FP32 inverse Jacobian until
 // the step is below newton_tol.  Returns the double-float xi in zd; a full
 // FP64 Newton is the (out-of-line) fallback.
-// Xs: optional copy of the element's FP32 nodes, high parts [3][G^3], then the
-// low parts from the next 16-byte boundary (read with generic loads when SH).
-template <int G, int SS = 0, bool SH = false>
+template <int G>
 __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, int e,
                                           const df* xd, const float* guess, df* zd, int& it32,
-                                          int& it64, float* sb = nullptr,
-                                          const float* Xs = nullptr) {
-  constexpr int G3 = G * G * G;
-  const float* X32 = Xs ? Xs : m.xg32 + (size_t)e * 3 * G3;
-  const float* X32l = Xs ? Xs + ((3 * G3 + 3) & ~3) : m.xg32lo + (size_t)e * 3 * G3;
-  const int tm = __ldg(m.tmask + e);
+                                          int& it64) {
+  const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
+  const float* Ml = m.monolo + (size_t)e * 3 * Mono<G>::CS;
+  const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
   float z[3] = {guess[0], guess[1], guess[2]};
   float Ji[9];
   bool have = false;
   #pragma unroll 1
   for (int it = 0; it < 8; ++it) {
     float chi[3], J[9], r[3], d[3];
-    map_j32<G, SS, SH>(X32, z, tm, k, chi, J, sb);
+    map_j32<G>(Mh, z, tm, chi, J);
     if (!inv3(J, Ji)) break;
     have = true;
 #pragma unroll
@@ -722,21 +282,29 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
     const float tol = (float)k.newton_tol;
     // Each step needs the residual at the current iterate.  The first is the
     // double-float residual at the FP32 iterate z.  After a first step d with
-    // |d| <= 4e-7 the next residual is r(z) + [chi(z - d) - chi(z)], the
-    // bracket an exact FP32 increment (it carries ~1e-7 of a term of size
-    // |J d|, far below the tolerance); later residuals are double-float again.
+    // |d| <= 4e-7 the next residual is r(z) + [chi(z - d) - chi(z)], and the
+    // bracket is -J(z - d/2) d up to terms of third order in d: FP32 gives it
+    // to ~1e-7 of a term of size |J d|, far below the tolerance.  Later
+    // residuals are double-float again, at the iterate's high part plus J
+    // times its low part.
     float rp[3] = {0.f, 0.f, 0.f}, dz[3] = {0.f, 0.f, 0.f};
     bool inc = false;
 #pragma unroll 1
     for (int it = 0; it < 6; ++it) {
-      float r[3], d[3];
-      if (inc) {
-        float dchi[3];
-        map_inc32<G, SH, SS>(X32, z, dz, tm, k, dchi, sb);
+      float r[3], d[3], zm[3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) r[q] = rp[q] + dchi[q];
-      } else {
-        resid_df<G, SS, SH>(X32, X32l, zd, tm, xd, k, r, sb);
+      for (int q = 0; q < 3; ++q) zm[q] = inc ? fmaf(0.5f, dz[q], z[q]) : zd[q].hi;
+      if (!inc) resid_df<G>(Mh, Ml, zm, tm, xd, rp);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) r[q] = rp[q];
+      if (it > 0) {
+        float chi[3], J[9], Jd[3];
+        const float by[3] = {inc ? dz[0] : zd[0].lo, inc ? dz[1] : zd[1].lo,
+                             inc ? dz[2] : zd[2].lo};
+        map_j32<G>(Mh, zm, tm, chi, J);
+        matvec3(J, by, Jd);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) r[q] += Jd[q];
       }
       matvec3(Ji, r, d);
 #pragma unroll
@@ -760,7 +328,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
     xi[q] = have ? df_to_double(zd[q]) : (double)guess[q];
   }
   if (!(tmax3(xi[0], xi[1], xi[2]) <= 4.0)) xi[0] = xi[1] = xi[2] = 0.0;
-  const bool ok = newton64_cold<G>(m.xg64 + (size_t)e * 3 * G3, xl, xi, k, it64);
+  const bool ok = newton64_cold<G>(m.xg64 + (size_t)e * 3 * G * G * G, xl, xi, k, it64);
 #pragma unroll
   for (int q = 0; q < 3; ++q) zd[q] = df_from_double(xi[q]);
   return ok;
@@ -784,24 +352,24 @@ __device__ __forceinline__ bool newton_mixed(const DevMesh& m, const DevConsts& 
 // interpolation of rho and rho u (Eq. part_interpolation), sum-factorised
 // ---------------------------------------------------------------------------
 
-// 1: the FP32 interpolation at N = 5 takes two variables per pass (their row
-// loads independent: twice the loads in flight; +5 % at the 64^3 workload)
-#ifndef PT_INTERP_V2
-#define PT_INTERP_V2 1
-#endif
-template <int NP, typename T, bool SH = false, int SS = 0>
+// FP32 at N = 5 takes two variables per pass (their row loads independent:
+// twice the loads in flight; +5 % at the 64^3 workload).  SS > 0: the
+// third-direction basis and the results, indexed by the rolled loops, go
+// through this thread's column of a [kScratchRows][SS] shared array at sb
+// instead of through local memory.
+constexpr int kScratchRows = 12;
+template <int NP, typename T, int SS = 0>
 __device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, const T* l2,
                                         const T* l3, T* out, float* sb = nullptr) {
   constexpr int N3 = NP * NP * NP;
-#if PT_INTERP_V2
   // two variables per pass: their row loads are independent, which doubles
   // the loads in flight per iteration
   if constexpr (std::is_same<T, float>::value && NP == 6) {
-    // rows kScratchOut + kk: l3; kScratchOut + NP + v: the results
-    constexpr bool kS = SS > 0 && PT_SMEM_OUT;
+    // rows kk: l3; NP + v: the results
+    constexpr bool kS = SS > 0;
     if constexpr (kS) {
 #pragma unroll
-      for (int kk = 0; kk < NP; ++kk) sb[(kScratchOut + kk) * SS] = l3[kk];
+      for (int kk = 0; kk < NP; ++kk) sb[kk * SS] = l3[kk];
     }
 #pragma unroll 1
     for (int v = 0; v < 4; v += 2) {
@@ -815,8 +383,8 @@ __device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, c
         for (int j = 0; j < NP; j += 2) {
           const float4* qa = reinterpret_cast<const float4*>(Ua + NP * (j + NP * kk));
           const float4* qb = reinterpret_cast<const float4*>(Ub + NP * (j + NP * kk));
-          const float4 a0 = ldx<SH>(qa), a1 = ldx<SH>(qa + 1), a2 = ldx<SH>(qa + 2);
-          const float4 b0 = ldx<SH>(qb), b1 = ldx<SH>(qb + 1), b2 = ldx<SH>(qb + 2);
+          const float4 a0 = __ldg(qa), a1 = __ldg(qa + 1), a2 = __ldg(qa + 2);
+          const float4 b0 = __ldg(qb), b1 = __ldg(qb + 1), b2 = __ldg(qb + 2);
           const float ra0[6] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y};
           const float ra1[6] = {a1.z, a1.w, a2.x, a2.y, a2.z, a2.w};
           const float rb0[6] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y};
@@ -834,13 +402,13 @@ __device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, c
           tb = fmaf(sb0, l2[j], tb);
           tb = fmaf(sb1, l2[j + 1], tb);
         }
-        const float lk = kS ? sb[(kScratchOut + kk) * SS] : l3[kk];
+        const float lk = kS ? sb[kk * SS] : l3[kk];
         acca = fmaf(ta, lk, acca);
         accb = fmaf(tb, lk, accb);
       }
       if constexpr (kS) {
-        sb[(kScratchOut + NP + v) * SS] = acca;
-        sb[(kScratchOut + NP + 1 + v) * SS] = accb;
+        sb[(NP + v) * SS] = acca;
+        sb[(NP + 1 + v) * SS] = accb;
       } else {
         out[v] = acca;
         out[v + 1] = accb;
@@ -848,15 +416,10 @@ __device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, c
     }
     if constexpr (kS) {
 #pragma unroll
-      for (int v = 0; v < 4; ++v) out[v] = sb[(kScratchOut + NP + v) * SS];
+      for (int v = 0; v < 4; ++v) out[v] = sb[(NP + v) * SS];
     }
     return;
   }
-#endif
-  // FP32 rows of 6 nodes: two rows (48 bytes, 16-byte aligned at even rows
-  // since every variable block is a multiple of 16 bytes) in three 16-byte
-  // loads; rows of 4 or 8 nodes in 16-byte loads
-  constexpr bool kPair = std::is_same<T, float>::value && NP == 6;
 #pragma unroll 1
   for (int v = 0; v < 4; ++v) {
     const T* Uv = Ue + v * N3;
@@ -864,56 +427,35 @@ __device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, c
 #pragma unroll 1
     for (int kk = 0; kk < NP; ++kk) {
       T t2 = T(0);
-      if constexpr (kPair) {
 #pragma unroll
-        for (int j = 0; j < NP; j += 2) {
-          const float4* q = reinterpret_cast<const float4*>(Uv + NP * (j + NP * kk));
-          const float4 q0 = ldx<SH>(q), q1 = ldx<SH>(q + 1), q2 = ldx<SH>(q + 2);
-          const float r0[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
-          const float r1[6] = {q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
-          T t1 = T(0), u1 = T(0);
+      for (int j = 0; j < NP; ++j) {
+        const T* row = Uv + NP * (j + NP * kk);
+        T t1 = T(0);
+        if constexpr (std::is_same<T, float>::value && NP % 4 == 0) {
 #pragma unroll
-          for (int i = 0; i < NP; ++i) t1 = tfma((T)r0[i], l1[i], t1);
-#pragma unroll
-          for (int i = 0; i < NP; ++i) u1 = tfma((T)r1[i], l1[i], u1);
-          t2 = tfma(t1, l2[j], t2);
-          t2 = tfma(u1, l2[j + 1], t2);
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-          const T* row = Uv + NP * (j + NP * kk);
-          T t1 = T(0);
-          if constexpr (std::is_same<T, float>::value && NP % 4 == 0) {
-#pragma unroll
-            for (int i = 0; i < NP; i += 4) {
-              const float4 q = ldx<SH>(reinterpret_cast<const float4*>(row + i));
-              t1 = tfma((T)q.x, l1[i], t1);
-              t1 = tfma((T)q.y, l1[i + 1], t1);
-              t1 = tfma((T)q.z, l1[i + 2], t1);
-              t1 = tfma((T)q.w, l1[i + 3], t1);
-            }
-          } else if constexpr (std::is_same<T, float>::value && NP % 2 == 0) {
-            float rv[NP];
-            load_row<NP, SH>(reinterpret_cast<const float*>(row), rv);
-#pragma unroll
-            for (int i = 0; i < NP; ++i) t1 = tfma((T)rv[i], l1[i], t1);
-          } else {
-#pragma unroll
-            for (int i = 0; i < NP; ++i) t1 = tfma(ldx<SH>(row + i), l1[i], t1);
+          for (int i = 0; i < NP; i += 4) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(row + i));
+            t1 = tfma((T)q.x, l1[i], t1);
+            t1 = tfma((T)q.y, l1[i + 1], t1);
+            t1 = tfma((T)q.z, l1[i + 2], t1);
+            t1 = tfma((T)q.w, l1[i + 3], t1);
           }
-          t2 = tfma(t1, l2[j], t2);
+        } else if constexpr (std::is_same<T, float>::value && NP % 2 == 0) {
+#pragma unroll
+          for (int i = 0; i < NP; i += 2) {
+            const float2 q = __ldg(reinterpret_cast<const float2*>(row + i));
+            t1 = tfma((T)q.x, l1[i], t1);
+            t1 = tfma((T)q.y, l1[i + 1], t1);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < NP; ++i) t1 = tfma(__ldg(row + i), l1[i], t1);
         }
+        t2 = tfma(t1, l2[j], t2);
       }
-#if PT_PICK_INTERP
-      acc = tfma(t2, pick<NP>(l3, kk), acc);
-    }
-    put<4>(out, v, acc);
-#else
       acc = tfma(t2, l3[kk], acc);
     }
     out[v] = acc;
-#endif
   }
 }
 

@@ -42,7 +42,8 @@ struct DevMesh {
   int g;                  // NGeo + 1
   const double* xg64;     // [E][g^3][3]   nodes - ce
   const float* xg32;      // [E][3][g^3]   nodes - ce, FP32, coordinate-major
-  const float* xg32lo;    // [E][3][g^3]   (nodes - ce) - xg32: low parts of a double-float copy
+  const float* mono;      // [E][3][CS]    monomial coefficients of nodes - ce (pt_map.cuh),
+  const float* monolo;    //               high and low FP32 parts
   const double* ce;       // [E][3]
   const float* tri;       // [E][12]       trilinear centre (3) and inverse Jacobian (9)
   const int* tmask;       // [E]           bit q: coordinate q is trilinear in xi (8-corner form)
@@ -60,7 +61,6 @@ struct DevMesh {
 struct DevConsts {
   double gn[PT_MAXG], gw[PT_MAXG];   // geometry nodes / barycentric weights
   float gn32[PT_MAXG], gw32[PT_MAXG];
-  float gn_hi[PT_MAXG], gn_lo[PT_MAXG], gw_hi[PT_MAXG], gw_lo[PT_MAXG];  // double-float copies
   double sn[PT_MAXN], sw[PT_MAXN];   // solution nodes / barycentric weights
   float sn32[PT_MAXN], sw32[PT_MAXN];
   double sq[PT_MAXN];                // quadrature weights of the solution nodes
@@ -168,8 +168,6 @@ struct StageArgs {
   int* hits;              // [n]
   unsigned* st;           // [n] status bits
   float* guess;           // [3][n] learned start (MLP) or null
-  float* xih;             // FP32 mode, split stage: [3][n] converged xi, double-float
-  float* xil;
   unsigned* list;         // [n] listed positions (| 1 << 31: walk only)
   unsigned* count;        // entries in list
   unsigned* count_next;   // the next stage's counter (cleared by this stage)

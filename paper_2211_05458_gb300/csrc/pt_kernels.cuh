@@ -165,7 +165,7 @@ __device__ __noinline__ void saffman_force(const DevMesh& m, const DevConsts& k,
   if constexpr (std::is_same<T, float>::value) {
     const float xf[3] = {(float)xi[0], (float)xi[1], (float)xi[2]};
     float chi[3];
-    map_j32<G>(m.xg32 + (size_t)e * 3 * G3, xf, __ldg(m.tmask + e), k, chi, J);
+    map_j32<G>(m.mono + (size_t)e * 3 * Mono<G>::CS, xf, __ldg(m.tmask + e), chi, J);
   } else {
     double chi[3];
     map64<G, true>(m.xg64 + (size_t)e * 3 * G3, xi, k, chi, J);
@@ -1356,30 +1356,6 @@ struct Family {
     }
     return (int)cudaGetLastError();
   }
-  // dynamic shared memory of k_stage_f32: the warp slots (blocks of 128 threads)
-  template <int NP>
-  static constexpr int stage_dyn_smem() {
-    if constexpr (F64)
-      return 0;
-    else
-      return UStage<NP>::ok ? 0 : WSlot<G, NP>::bytes;
-  }
-  // allows the dynamic shared memory above 48 KB per block; set once per
-  // instantiation, before the first occupancy query or launch
-  template <int NP>
-  static void stage_smem_attr() {
-    constexpr int dyn = stage_dyn_smem<NP>();
-    if constexpr (dyn > 0) {
-      static bool attr = false;
-      if (!attr) {
-        cudaFuncSetAttribute(k_stage_f32<G, NP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             dyn);
-        cudaFuncSetAttribute(k_stage_f32<G, NP, kMlp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             dyn);
-        attr = true;
-      }
-    }
-  }
   template <int NP>
   static int staged(int op, const StageArgs& a, const DevParticles& p, const int* perm, int grid,
                     int block, cudaStream_t s) {
@@ -1390,19 +1366,10 @@ struct Family {
       case PT_SOP_STAGE:
         if constexpr (F64) {
           k_stage_f64<G, NP><<<grid, block, 0, s>>>(a);
-        } else if (PT_STAGE_SPLIT && !UStage<NP>::ok) {
-          if (kMlp && a.k.guess == PT_GUESS_MLP)
-            k_locate_f32<G, kMlp><<<grid, block, 0, s>>>(a);
-          else
-            k_locate_f32<G, false><<<grid, block, 0, s>>>(a);
-          k_advance_f32<G, NP><<<grid, block, 0, s>>>(a);
+        } else if (kMlp && a.k.guess == PT_GUESS_MLP) {
+          k_stage_f32<G, NP, kMlp><<<grid, block, 0, s>>>(a);
         } else {
-          constexpr int dyn = stage_dyn_smem<NP>();
-          stage_smem_attr<NP>();
-          if (kMlp && a.k.guess == PT_GUESS_MLP)
-            k_stage_f32<G, NP, kMlp><<<grid, block, dyn, s>>>(a);
-          else
-            k_stage_f32<G, NP, false><<<grid, block, dyn, s>>>(a);
+          k_stage_f32<G, NP, false><<<grid, block, 0, s>>>(a);
         }
         break;
       case PT_SOP_TRACK:
@@ -1454,15 +1421,8 @@ struct Family {
     int nb = 0;
     if constexpr (F64) {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage_f64<G, NP>, block, 0);
-    } else if (PT_STAGE_SPLIT && !UStage<NP>::ok) {
-      int nl = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_advance_f32<G, NP>, block, 0);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nl, k_locate_f32<G, false>, block, 0);
-      nb = nb < nl ? nb : nl;
     } else {
-      stage_smem_attr<NP>();
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage_f32<G, NP, false>, block,
-                                                    stage_dyn_smem<NP>());
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage_f32<G, NP, false>, block, 0);
     }
     return nb;
   }
