@@ -344,7 +344,8 @@ struct MonoBasis {
 
 template <int G>
 __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tmask, int nelem,
-                       const MonoBasis V, float* __restrict__ hi, float* __restrict__ lo) {
+                       const MonoBasis V, float* __restrict__ hi, float* __restrict__ lo,
+                       float* __restrict__ curv) {
   constexpr int G3 = G * G * G, AP = Mono<G>::AP, CS = Mono<G>::CS;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * nelem) return;
@@ -356,6 +357,13 @@ __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tm
     h[q] = (float)v;
     l[q] = (float)(v - (double)h[q]);
   };
+  // sum |M| n (n - 1) 1.1^n, n = a + b + c: |chi_r''(D, D)| <= this |D|^2
+  double sum = 0.0;
+  auto bound = [&](int n, double v) {
+    double w = fabs(v) * n * (n - 1);
+    for (int q = 0; q < n; ++q) w *= 1.1;
+    sum += w;
+  };
   if ((tmask[e] >> r) & 1) {  // 8 coefficients of the corner interpolant
     for (int q = 0; q < 8; ++q) {
       double v = 0.0;
@@ -365,8 +373,10 @@ __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tm
         v += (__popc(q & ~w) & 1) ? -xv : xv;
       }
       put(q, 0.125 * v);
+      bound(__popc(q), 0.125 * v);
     }
     for (int q = 8; q < CS; ++q) h[q] = l[q] = 0.f;
+    curv[4 * (size_t)e + r] = (float)(sum * (1.0 + 1e-6));
     return;
   }
   double T[G3];
@@ -385,7 +395,11 @@ __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tm
   for (int q = 0; q < CS; ++q) h[q] = l[q] = 0.f;
   for (int c = 0; c < G; ++c)
     for (int b = 0; b < G; ++b)
-      for (int a = 0; a < G; ++a) put(AP * (c + G * b) + a, T[a + G * (b + G * c)]);
+      for (int a = 0; a < G; ++a) {
+        put(AP * (c + G * b) + a, T[a + G * (b + G * c)]);
+        bound(a + b + c, T[a + G * (b + G * c)]);
+      }
+  curv[4 * (size_t)e + r] = (float)(sum * (1.0 + 1e-6));
 }
 
 static int mono_floats(int g) {
@@ -409,10 +423,10 @@ static cudaError_t launch_mono(pt_ctx* c) {
   }
   const int nb = (3 * c->nelem + 127) / 128;
   switch (c->g) {
-    case 2: k_mono<2><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
-    case 3: k_mono<3><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
-    case 4: k_mono<4><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
-    default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo); break;
+    case 2: k_mono<2><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
+    case 3: k_mono<3><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
+    case 4: k_mono<4><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
+    default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
   }
   const cudaError_t err = cudaGetLastError();
   return err ? err : cudaStreamSynchronize(c->stream);
@@ -649,6 +663,8 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_monolo = dmalloc<float>(cc, nmono, &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
+  c->d_curv = dmalloc<float>(cc, 4 * (size_t)E, &err);
+  if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_ce = dmalloc<double>(cc, ce.size(), &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_tri = dmalloc<float>(cc, tri.size(), &err);
@@ -733,6 +749,8 @@ static void fill_consts(const pt_ctx* c, DevConsts& k) {
   k.newton_tol = c->cfg.newton_tol;
   k.band_ref = c->cfg.band_ref;
   k.band_x = c->cfg.band_x;
+  k.band_ref32 = (float)c->cfg.band_ref;
+  k.band_x32 = (float)c->cfg.band_x;
   k.lost_tol = c->cfg.lost_tol;
   k.drag_law = c->cfg.drag_law;
   k.lift = c->cfg.lift;
@@ -760,6 +778,7 @@ static DevMesh dev_mesh(const pt_ctx* c) {
   m.xg32 = c->d_xg32;
   m.mono = c->d_mono;
   m.monolo = c->d_monolo;
+  m.curv = c->d_curv;
   m.ce = c->d_ce;
   m.tri = c->d_tri;
   m.tmask = c->d_tmask;
@@ -1033,7 +1052,7 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   bytes += 3 * al(3 * rs * nn) + al(rs * nn);         // v, kx, kv, d
   bytes += al((f64 ? 24 : 24) * nn);                  // xe
   bytes += f64 ? 0 : al(12 * nn);                     // guess
-  bytes += 4 * al(4 * nn) + 256;                      // e, hits, st, list, counters
+  bytes += (f64 ? 4 : 5) * al(4 * nn) + 256;          // e, hits, st, list(s), counters
   if (c->state_cap < n || !c->d_state) {
     if (c->d_state) cudaFree(c->d_state);
     c->d_state = nullptr;
@@ -1068,8 +1087,8 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   a.hits = (int*)take(4 * nn);
   a.st = (unsigned*)take(4 * nn);
   a.list = (unsigned*)take(4 * nn);
-  a.count = (unsigned*)b;
-  a.count_next = a.count + 1;
+  a.list2 = f64 ? nullptr : (unsigned*)take(4 * nn);
+  a.count = (unsigned*)b;  // four counters
   return PT_OK;
 }
 
@@ -1079,9 +1098,9 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
 // Launch shapes of the staged schedule for n particles.
 struct StagedLaunch {
   bool f64 = false, mlp = false;
-  int np = 0, grid = 1, block = 128, gmove = 1, gtrack = 1, gguess = 1;
+  int np = 0, grid = 1, block = 128, gmove = 1, gtrack = 1, gexact = 1, gguess = 1;
   DevParticles dp{};
-  unsigned* ctr = nullptr;  // two list counters, used by alternate stages
+  unsigned* ctr = nullptr;  // two counters per list, used by alternate stages
 };
 
 static pt_status staged_prepare(pt_ctx* c, const pt_particles* p, double dt, StageArgs& a,
@@ -1103,7 +1122,9 @@ static pt_status staged_prepare(pt_ctx* c, const pt_particles* p, double dt, Sta
   const int occ = max_active_stage(c->g, L.f64, L.np, L.block);
   L.grid = grid_for(c, n, L.block, occ);
   L.gmove = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)c->nsm * 8));
-  L.gtrack = c->nsm * 4;
+  // list kernels: a few thousand entries per stage at most shapes, latency-bound
+  L.gtrack = c->nsm * (L.f64 ? 4 : 12);
+  L.gexact = c->nsm * 8;
   L.gguess = (int)std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, (int64_t)c->nsm * 4));
   L.ctr = a.count;
   return PT_OK;
@@ -1125,20 +1146,29 @@ static int staged_stage(pt_ctx* c, StageArgs& a, const StagedLaunch& L, int st, 
   a.stage = st;
   a.count = L.ctr + (k & 1);
   a.count_next = L.ctr + ((k + 1) & 1);
-  // each kernel between an event pair of its kind when profiling
-  auto timed = [&](int kind, int op, int g, int b) {
+  a.count2 = L.ctr + 2 + (k & 1);
+  a.count2_next = L.ctr + 2 + ((k + 1) & 1);
+  auto launch = [&](int op, int g, int b) {
+    c->launches += 1;
+    return launch_staged(c->g, L.f64, L.np, op, a, L.dp, c->d_perm, g, b, c->stream);
+  };
+  // kernels between an event pair of their kind when profiling
+  auto timed = [&](int kind, auto&& body) {
     cudaEvent_t q0 = c->profile ? take_event(c, kind) : nullptr;
     cudaEvent_t q1 = c->profile ? take_event(c, kind) : nullptr;
     if (q0) cudaEventRecord(q0, c->stream);
-    const int r = launch_staged(c->g, L.f64, L.np, op, a, L.dp, c->d_perm, g, b, c->stream);
+    const int r = body();
     if (q1) cudaEventRecord(q1, c->stream);
-    c->launches += 1;
     return r;
   };
   int rc = 0;
-  if (L.mlp) rc = timed(2, PT_SOP_GUESS, L.gguess, 128);
-  if (!rc) rc = timed(1, PT_SOP_STAGE, L.grid, L.block);
-  if (!rc) rc = timed(3, PT_SOP_TRACK, L.gtrack, 128);
+  if (L.mlp) rc = timed(2, [&] { return launch(PT_SOP_GUESS, L.gguess, 128); });
+  if (!rc) rc = timed(1, [&] { return launch(PT_SOP_STAGE, L.grid, L.block); });
+  if (!rc)
+    rc = timed(3, [&] {
+      const int r = launch(PT_SOP_TRACK, L.gtrack, 128);
+      return r || L.f64 ? r : launch(PT_SOP_EXACT, L.gexact, 32);
+    });
   return rc;
 }
 
@@ -1156,7 +1186,7 @@ static pt_status push_staged(pt_ctx* c, const pt_particles* p, int32_t nsteps, d
   StagedLaunch L;
   pt_status s = staged_prepare(c, p, dt, a, L);
   if (s) return s;
-  CK(cudaMemsetAsync(L.ctr, 0, 2 * sizeof(unsigned), c->stream));
+  CK(cudaMemsetAsync(L.ctr, 0, 4 * sizeof(unsigned), c->stream));
   const int chunk = c->cfg.rebin_every > 0 ? c->cfg.rebin_every : 10;
   int k = 0;
   for (int s0 = 0; s0 < nsteps; s0 += chunk) {
@@ -1273,7 +1303,7 @@ pt_status pt_push_stage(pt_ctx* c, const pt_particles* p, int32_t stage, double 
   int rc = 0;
   if (n > 0) {
     if (stage == 0) {
-      CK(cudaMemsetAsync(L.ctr, 0, 2 * sizeof(unsigned), c->stream));
+      CK(cudaMemsetAsync(L.ctr, 0, 4 * sizeof(unsigned), c->stream));
       rc = staged_begin(c, p, a, L);
     }
     if (!rc) rc = staged_stage(c, a, L, stage, stage);

@@ -25,12 +25,6 @@
 #ifndef PT_FACE_SCREEN
 #define PT_FACE_SCREEN 1
 #endif
-// 1 (FP32 mode): an internal or periodic crossing that the FP32 screen finds
-// unambiguous is taken without the FP64 solve (see track_slow)
-#ifndef PT_FP32_DECIDE
-#define PT_FP32_DECIDE 1
-#endif
-
 namespace pt {
 
 template <typename T>
@@ -246,18 +240,19 @@ __device__ __noinline__ bool newton64_cold(const double* X64, const double* xl, 
 // Mixed-precision Newton on a double-float local position xd (relative to the
 // element centre): FP32 iterations (chi and J in FP32) until the step is below
 // 1e-5, then double-float residuals with the last FP32 inverse Jacobian until
-// the step is below newton_tol.  Returns the double-float xi in zd; a full
-// FP64 Newton is the (out-of-line) fallback.
+// the step is below newton_tol.  Returns the double-float xi in zd and, unless
+// the (out-of-line) fallback of a full FP64 Newton was taken (jok false), the
+// inverse Jacobian at xi to ~1e-5 in Ji.
 template <int G>
 __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, int e,
                                           const df* xd, const float* guess, df* zd, int& it32,
-                                          int& it64) {
+                                          int& it64, float* Ji, bool& jok) {
   const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
   const float* Ml = m.monolo + (size_t)e * 3 * Mono<G>::CS;
   const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
   float z[3] = {guess[0], guess[1], guess[2]};
-  float Ji[9];
   bool have = false;
+  jok = true;
   #pragma unroll 1
   for (int it = 0; it < 8; ++it) {
     float chi[3], J[9], r[3], d[3];
@@ -321,6 +316,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
     }
   }
   // fallback: full FP64 Newton
+  jok = false;
   double xl[3], xi[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -332,6 +328,15 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
 #pragma unroll
   for (int q = 0; q < 3; ++q) zd[q] = df_from_double(xi[q]);
   return ok;
+}
+
+template <int G>
+__device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, int e,
+                                          const df* xd, const float* guess, df* zd, int& it32,
+                                          int& it64) {
+  float Ji[9];
+  bool jok;
+  return newton_df<G>(m, k, e, xd, guess, zd, it32, it64, Ji, jok);
 }
 
 // As newton_df for a local position in FP64 (xl) and a FP64 result.
@@ -1191,6 +1196,222 @@ __device__ __noinline__ void mortar_enter(const DevMesh& m, const DevConsts& k, 
   anew = ka;
 }
 
+// Bound on how far xi(x + dx) can be from xi(x) + D, D = Ji dx, along the
+// straight segment dx: with the second derivatives of chi_r bounded by S_r
+// (DevMesh::curv) and K_d = sum_j |Ji_dj| S_j / 2, |xi - xi_lin|_d <= 2 K_d |D|^2
+// while K |D| <= 1/8 (else the bound is not used: returns false).  marg[d] is
+// that bound plus the distance band_x in reference units plus 1e-5 for the FP32
+// rounding of xi and Ji, curv the largest of the curvature parts.
+__device__ __forceinline__ bool xi_margin(const DevMesh& m, int e, const float* Ji,
+                                          const float* dx, float bx, float* D, float* marg,
+                                          float& curv) {
+  const float4 S = __ldg(reinterpret_cast<const float4*>(m.curv) + e);
+  matvec3(Ji, dx, D);
+  const float a = tmax3(D[0], D[1], D[2]);
+  const float c[3] = {S.x * a * a, S.y * a * a, S.z * a * a};
+  curv = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float j0 = fabsf(Ji[3 * d]), j1 = fabsf(Ji[3 * d + 1]), j2 = fabsf(Ji[3 * d + 2]);
+    const float q = j0 * c[0] + j1 * c[1] + j2 * c[2];
+    curv = fmaxf(curv, q);
+    marg[d] = q + (j0 + j1 + j2) * bx + 1e-5f;
+  }
+  return curv <= 0.25f * a;
+}
+
+// True only if the stage segment from xi (inside element e) along dx cannot come
+// within the bands of any face: its linearised path and the bound above stay
+// inside.  Ji: the inverse Jacobian at xi.  Much sharper than the faces' slabs,
+// which are as thick as a face is curved (0.85 % of the 32^3 channel's segments
+// touch a slab, 0.12 % cross a face), and it needs 16 bytes of the element
+// instead of 192.
+__device__ __forceinline__ bool stays_inside(const DevMesh& m, int e, const float* xi,
+                                             const float* Ji, const float* dx, float bx) {
+  float D[3], marg[3], curv;
+  bool in = xi_margin(m, e, Ji, dx, bx, D, marg, curv);
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    in = in && fmaxf(fabsf(xi[d]), fabsf(xi[d] + D[d])) <= 1.f - marg[d];
+  return in;
+}
+
+// One Newton step d on F(s, t, alpha) = chi(s, t on face f) - (x + alpha td) = 0
+// from the Jacobian in FP32 and the double-float residual of the inverse map
+// (error ~1e-14 of the element); x a double-float offset, td the unit
+// direction.  cosr: the cosine between the ray and the face normal there.
+// False if the Jacobian is singular.
+template <int G>
+__device__ __forceinline__ bool face_step(const DevMesh& m, int e, int tm, int f, const df* x,
+                                          const float* td, float s, float t, float al, float* d,
+                                          float& cosr) {
+  const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
+  const int q = f >> 1;
+  const float w = (f & 1) ? 1.f : -1.f;
+  // xi_q = -1 or +1, s and t along the two other directions in order
+  const float xi[3] = {q == 0 ? w : s, q == 1 ? w : (q == 0 ? s : t), q == 2 ? w : t};
+  float chi[3], J[9], A[9], Ai[9], F[3];
+  map_j32<G>(Mh, xi, tm, chi, J);
+  df xa[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    A[3 * r] = q == 0 ? J[3 * r + 1] : J[3 * r];
+    A[3 * r + 1] = q == 2 ? J[3 * r + 1] : J[3 * r + 2];
+    A[3 * r + 2] = -td[r];
+    df p;
+    two_prod(al, td[r], p.hi, p.lo);
+    xa[r] = df_add(x[r], p);
+  }
+  if (!inv3(A, Ai)) return false;
+  resid_df<G>(Mh, m.monolo + (size_t)e * 3 * Mono<G>::CS, xi, tm, xa, F);
+  // row 3 of Ai is -n / (n . td), n the face normal p_s x p_t
+  cosr = 1.f / sqrtf(Ai[6] * Ai[6] + Ai[7] * Ai[7] + Ai[8] * Ai[8]);
+  matvec3(Ai, F, d);
+  return true;
+}
+
+// FP32 pass of the tracking (FP32 mode): the stage segment xd -> xe (double-
+// float offsets from the centre of element e) in reference space.  In the
+// current element the end point's xi is found by the inverse map, and the
+// segment's path is xi - (1 - tau) D up to the bound of xi_margin.  Only faces
+// that the path can come to within the bands are intersected: the linear path
+// gives the start, two Newton steps with the double-float residual leave alpha
+// good to ~1e-13 of the element over the cosine to the face, and acceptance
+// and the near-face bands are decided with margins (tb, 2e-6 in s and t) four
+// orders above that.  The smallest accepted alpha wins; an internal or
+// periodic face leads to the next element, the position is the segment's end.
+// A wall, open or mortar face that is hit, a path nearly parallel to a face it
+// may reach, a quantity within the margin of its threshold and two crossings
+// within the margin return false with nothing changed, and track_slow
+// intersects the faces in FP64.
+template <int G>
+__device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, int& e_io, df* xd,
+                                          const df* xe, unsigned& st, int& it32, int& it64,
+                                          TrackCounters& tc) {
+  int e = e_io, cross = 0, fin = -1;
+  unsigned bits = 0u;
+  float dx[3], td[3], a0 = 0.f;
+  df x[3] = {xe[0], xe[1], xe[2]};      // the segment's ends in the current element's frame
+  df x0[3] = {xd[0], xd[1], xd[2]};
+  double xg[3] = {0.0, 0.0, 0.0}, xs[3] = {0.0, 0.0, 0.0};  // global, once it has crossed
+#pragma unroll
+  for (int r = 0; r < 3; ++r) dx[r] = (xe[r].hi - xd[r].hi) + (xe[r].lo - xd[r].lo);
+  const float L = sqrtf(dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2]);
+  if (!(L > 0.f)) return false;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) td[r] = dx[r] / L;
+  const float bx = k.band_x32, br = k.band_ref32, ext = 1.f + 2.f * bx / L;
+#pragma unroll 1
+  while (true) {
+    const float xf[3] = {x[0].hi, x[1].hi, x[2].hi};
+    const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
+    float g[3], Ji[9], D[3], marg[3], curv;
+    df zd[3];
+    trilinear_guess(m, e, xf, g);
+    bool jok;
+    if (!newton_df<G>(m, k, e, x, g, zd, it32, it64, Ji, jok) || !jok) return false;
+    if (!xi_margin(m, e, Ji, dx, bx, D, marg, curv)) return false;
+    unsigned faces = 0u;
+    bool in = true;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float z1 = zd[d].hi, z0 = z1 - D[d];
+      if (fmaxf(z0, z1) > 1.f - marg[d]) faces |= 2u << (2 * d);
+      if (fminf(z0, z1) < -1.f + marg[d]) faces |= 1u << (2 * d);
+      in = in && fabsf(z1) <= 1.f;
+    }
+    if (fin >= 0) faces &= ~(1u << fin);
+    int pf = -1;
+    float pal = 0.f, ptb = 0.f;
+#pragma unroll 1
+    while (faces) {
+      const int f = __ffs(faces) - 1, q = f >> 1;
+      faces &= faces - 1u;
+      const float w = (f & 1) ? 1.f : -1.f;
+      const float Dq = q == 0 ? D[0] : (q == 1 ? D[1] : D[2]);
+      const float zq = q == 0 ? zd[0].hi : (q == 1 ? zd[1].hi : zd[2].hi);
+      // the path (and band_x beyond its ends) is monotone across the face, so
+      // that it meets the face once: slope Dq against the bend of the bound
+      if (!(fabsf(Dq) > fmaxf(2.f * ext * curv, 1e-2f * tmax3(D[0], D[1], D[2])))) return false;
+      const float u = (zq - w) / Dq;  // 1 - tau at the face
+      if (!(fabsf(u) < 4.f * ext)) continue;
+      float s = q == 0 ? zd[1].hi - u * D[1] : zd[0].hi - u * D[0];
+      float t = q == 2 ? zd[1].hi - u * D[1] : zd[2].hi - u * D[2];
+      float al = L - u * L, d[3], cosr = 0.f;
+#pragma unroll 1
+      for (int it = 0; it < 2; ++it) {
+        if (!face_step<G>(m, e, tm, f, x0, td, s, t, al, d, cosr)) return false;
+        s -= d[0];
+        t -= d[1];
+        al -= d[2];
+      }
+      if (!(cosr > 1e-3f) || !(fabsf(d[0]) < 1e-5f && fabsf(d[1]) < 1e-5f && fabsf(d[2]) < 1e-4f * (L + bx)))
+        return false;
+      const float Rmax = __ldg(m.slab + 48 * (size_t)e + 5);
+      const float mm = fmaxf(fabsf(s), fabsf(t)), tb = 1e-8f * (Rmax + L) / cosr;
+      const float om = mm - 1.f, da = al - a0, dL = L - al;
+      if (om > br + 2e-6f || da < -bx - tb || dL < -bx - tb) continue;
+      if (fabsf(om) <= 2e-6f || fabsf(fabsf(om) - br) <= 2e-6f || fabsf(da) <= tb ||
+          fabsf(dL) <= tb || fabsf(fabsf(da) - bx) <= tb || fabsf(fabsf(dL) - bx) <= tb)
+        return false;
+      const int bc = finfo_bc(__ldg(m.finfo + 6 * (size_t)e + f));
+      if (fabsf(om) < br || fabsf(da) < bx || fabsf(dL) < bx)
+        bits |= PT_ST_NEAR_FACE |
+                ((bc == PT_BC_WALL || bc == PT_BC_OPEN) ? (unsigned)PT_ST_NEAR_WALL : 0u);
+      if (om < 0.f && da > 0.f && dL > 0.f) {
+        if (!(bc == PT_BC_INTERNAL || bc == PT_BC_PERIODIC)) return false;
+        if (pf >= 0 && fabsf(al - pal) <= tb + ptb) return false;
+        if (pf < 0 || al < pal) {
+          pf = f;
+          pal = al;
+          ptb = tb;
+        }
+      }
+    }
+    if (pf < 0) {
+      if (!in) return false;
+      break;
+    }
+    if (cross + 1 >= k.max_cross || cross >= 8) return false;
+    if (!cross) {
+      const double* ce = m.ce + 3 * (size_t)e;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const double cr = __ldg(ce + r);
+        xs[r] = cr + df_to_double(xd[r]);
+        xg[r] = cr + df_to_double(xe[r]);
+      }
+    }
+    const int info = __ldg(m.finfo + 6 * (size_t)e + pf);
+    if (finfo_bc(info) == PT_BC_PERIODIC) {
+      const double* sh = m.shift + 18 * (size_t)e + 3 * pf;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        xs[r] += __ldg(sh + r);
+        xg[r] += __ldg(sh + r);
+      }
+    }
+    fin = finfo_nf(info);
+    e = __ldg(m.fnbr + 6 * (size_t)e + pf);
+    a0 = pal;
+    const double* cn = m.ce + 3 * (size_t)e;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const double cr = __ldg(cn + r);
+      x[r] = df_from_double(xg[r] - cr);
+      x0[r] = df_from_double(xs[r] - cr);
+    }
+    ++cross;
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) xd[r] = x[r];
+  e_io = e;
+  st |= bits;
+  tc.cross += cross;
+  ++tc.slow;
+  return true;
+}
+
 // CLIP: curved faces by Bezier clipping (a separate instantiation, so that the
 // default path carries none of its code)
 template <int G, typename R, bool CLIP>
@@ -1242,156 +1463,106 @@ __device__ __noinline__ void track_slow(const DevMesh& m, const DevConsts& k, in
     const float xlf[3] = {(float)xl[0], (float)xl[1], (float)xl[2]};
     double best = 1e300, bs = 0.0, bt = 0.0;
     int bf = -1;
-    // FP32 decision (FP32 mode): when exactly one face survives the screen,
-    // it is internal or periodic, and its only FP32 crossing lies clearly
-    // inside the face (max(|s|,|t|) < 1 - dl) and clearly inside the segment
-    // (by the screen's margin ta, ~100x the FP32 error) while its other roots
-    // are clearly outside, that crossing decides the exit face without the
-    // FP64 solve: the owner follows from the face alone, the position is the
-    // stage end point, and no near-face band can be met.  Otherwise the
-    // provisional faces are solved exactly in a second pass.
-    constexpr bool kFast = PT_FP32_DECIDE && PT_FACE_SCREEN && std::is_same<R, float>::value;
-    int pf = -1, npro = 0;
-    bool exact_seen = false;
-    float pa32 = 0.f, ps32 = 0.f, pt32 = 0.f;
-    unsigned redo = 0u;
 #pragma unroll 1
-    for (int pass = 0; pass < (kFast ? 2 : 1); ++pass) {
-      if (pass == 1 && (pf < 0 || (npro == 1 && !exact_seen))) break;
-#pragma unroll 1
-      for (int f = 0; f < 6; ++f) {
-        if (f == fin) continue;
-        if (pass == 1 && !((redo >> f) & 1u)) continue;
-        // slab prefilter (FP32, conservative: the margins cover its rounding)
-        const float* sl = m.slab + 48 * (size_t)e + 8 * f;
-        const float cosf_ = __ldg(sl) * tdf[0] + __ldg(sl + 1) * tdf[1] + __ldg(sl + 2) * tdf[2];
-        const float pa = __ldg(sl) * xlf[0] + __ldg(sl + 1) * xlf[1] + __ldg(sl + 2) * xlf[2];
-        const float pb = pa + Lf * cosf_;
-        if (fmaxf(pa, pb) < __ldg(sl + 3) || fminf(pa, pb) > __ldg(sl + 4)) continue;
-        const int info = __ldg(m.finfo + 6 * (size_t)e + f);
-        const int kind = finfo_kind(info);
-        // FP32 screen: skip the exact solve when every FP32 root is clearly
-        // outside the segment or the face (margins ~100x the FP32 error)
-        float fs[2], ft[2], fa[2];
-        bool ill = fabsf(cosf_) < 1e-2f;
-        if (PT_FACE_SCREEN) {
-          const float* Bf32 = m.bil32 + 72 * (size_t)e + 12 * f;
-          float B32[12];
+    for (int f = 0; f < 6; ++f) {
+      if (f == fin) continue;
+      // slab prefilter (FP32, conservative: the margins cover its rounding)
+      const float* sl = m.slab + 48 * (size_t)e + 8 * f;
+      const float cosf_ = __ldg(sl) * tdf[0] + __ldg(sl + 1) * tdf[1] + __ldg(sl + 2) * tdf[2];
+      const float pa = __ldg(sl) * xlf[0] + __ldg(sl + 1) * xlf[1] + __ldg(sl + 2) * xlf[2];
+      const float pb = pa + Lf * cosf_;
+      if (fmaxf(pa, pb) < __ldg(sl + 3) || fminf(pa, pb) > __ldg(sl + 4)) continue;
+      const int info = __ldg(m.finfo + 6 * (size_t)e + f);
+      const int kind = finfo_kind(info);
+      // FP32 screen: skip the exact solve when every FP32 root is clearly
+      // outside the segment or the face (margins ~100x the FP32 error)
+      float fs[2], ft[2], fa[2];
+      bool ill = fabsf(cosf_) < 1e-2f;
+      if (PT_FACE_SCREEN) {
+        const float* Bf32 = m.bil32 + 72 * (size_t)e + 12 * f;
+        float B32[12];
 #pragma unroll
-          for (int q = 0; q < 12; ++q) B32[q] = __ldg(Bf32 + q);
-          const int n32 = bilinear_roots_f32(B32, xlf, tdf, n1f, n2f, fs, ft, fa, ill);
-          const float ta = 1e-4f * (__ldg(sl + 5) + Lf) / fmaxf(fabsf(cosf_), 1e-2f) +
-                           4.f * (float)k.band_x;
-          const float a0f = (float)a0;
-          const float dl = fmaxf(1e-3f, 2.f * (float)k.band_ref);
-          bool any = ill, amb = ill;
-          int nin = 0, iin = 0;
-          #pragma unroll 1
-          for (int i = 0; i < n32 && !ill; ++i) {
-            if (kind == PT_FACE_CURVED &&
-                !curved_newton_f32<G>(m.xg32 + (size_t)e * 3 * G * G * G, f, xlf, tdf, k, fs[i],
-                                      ft[i], fa[i])) {
-              any = true;
-              amb = true;
-              break;
-            }
-            const float mm = fmaxf(fabsf(fs[i]), fabsf(ft[i]));
-            if (!(fa[i] < a0f - ta || fa[i] > Lf + ta || mm > 1.f + 1e-3f)) any = true;
-            if constexpr (kFast) {
-              const bool out = fa[i] < a0f - ta || fa[i] > Lf + ta || mm > 1.f + dl;
-              if (mm < 1.f - dl && fa[i] > a0f + ta && fa[i] < Lf - ta) {
-                ++nin;
-                iin = i;
-              } else if (!out) {
-                amb = true;
-              }
-            }
+        for (int q = 0; q < 12; ++q) B32[q] = __ldg(Bf32 + q);
+        const int n32 = bilinear_roots_f32(B32, xlf, tdf, n1f, n2f, fs, ft, fa, ill);
+        const float ta = 1e-4f * (__ldg(sl + 5) + Lf) / fmaxf(fabsf(cosf_), 1e-2f) +
+                         4.f * (float)k.band_x;
+        const float a0f = (float)a0;
+        bool any = ill;
+        #pragma unroll 1
+        for (int i = 0; i < n32 && !ill; ++i) {
+          if (kind == PT_FACE_CURVED &&
+              !curved_newton_f32<G>(m.xg32 + (size_t)e * 3 * G * G * G, f, xlf, tdf, k, fs[i],
+                                    ft[i], fa[i])) {
+            any = true;
+            break;
           }
-          if (!any) continue;
-          if constexpr (kFast) {
-            const int bcf = finfo_bc(info);
-            if (pass == 0 && !amb && nin == 1 && !(CLIP && kind == PT_FACE_CURVED) &&
-                (bcf == PT_BC_INTERNAL || bcf == PT_BC_PERIODIC)) {
-              ++npro;
-              pf = f;
-              pa32 = fa[iin];
-              ps32 = fs[iin];
-              pt32 = ft[iin];
-              redo |= 1u << f;
-              continue;
-            }
-          }
+          const float mm = fmaxf(fabsf(fs[i]), fabsf(ft[i]));
+          if (!(fa[i] < a0f - ta || fa[i] > Lf + ta || mm > 1.f + 1e-3f)) any = true;
         }
-        exact_seen = true;
-        const double* Bf = m.bil + 72 * (size_t)e + 12 * f;
-        double Bl[12];
+        if (!any) continue;
+      }
+      const double* Bf = m.bil + 72 * (size_t)e + 12 * f;
+      double Bl[12];
 #pragma unroll
-        for (int q = 0; q < 12; ++q) Bl[q] = __ldg(Bf + q);
-        constexpr int MR = CLIP ? 4 : 2;
-        double rs[MR], rt[MR], ra[MR];
-        int nr = 0;
-        const bool clip_all = CLIP && kind == PT_FACE_CURVED;
-        if constexpr (CLIP) {
-          if (clip_all)
-            nr = bezier_clip_roots<G>(X64, m.xg32 + (size_t)e * 3 * G * G * G, f, xl, td, n1, n2,
-                                      k, L, rs, rt, ra, MR);
-          else
-            nr = bilinear_roots(Bl, xl, td, n1, n2, rs, rt, ra);
-        } else {
+      for (int q = 0; q < 12; ++q) Bl[q] = __ldg(Bf + q);
+      constexpr int MR = CLIP ? 4 : 2;
+      double rs[MR], rt[MR], ra[MR];
+      int nr = 0;
+      const bool clip_all = CLIP && kind == PT_FACE_CURVED;
+      if constexpr (CLIP) {
+        if (clip_all)
+          nr = bezier_clip_roots<G>(X64, m.xg32 + (size_t)e * 3 * G * G * G, f, xl, td, n1, n2,
+                                    k, L, rs, rt, ra, MR);
+        else
           nr = bilinear_roots(Bl, xl, td, n1, n2, rs, rt, ra);
-        }
-        if (kind == PT_FACE_CURVED && !clip_all) {
-          // the curved face lies within dev of its bilinear patch: a bilinear
-          // crossing far beyond the segment cannot refine into one inside it
-          const double dev = (double)__ldg(sl + 6);
-          const double reach = 4.0 * dev / fmax((double)fabsf(cosf_), 0.05) + 2.0 * k.band_x;
-          int kk = 0;
-          #pragma unroll 1
-          for (int i = 0; i < nr; ++i) {
-            double s = rs[i], t = rt[i], al = ra[i];
-            if (!(fabs(s) < 2.0 && fabs(t) < 2.0)) continue;
-            if (al > L + reach || al < a0 - reach) continue;
-            if (curved_refine<G>(X64, m.xg32 + (size_t)e * 3 * G * G * G, f, xl, td, k, s, t,
-                                 al, L)) {
-              bool dup = false;
-              for (int j = 0; j < kk; ++j)
-                if (fabs(rs[j] - s) < 1e-10 && fabs(rt[j] - t) < 1e-10) dup = true;
-              if (!dup) {
-                rs[kk] = s;
-                rt[kk] = t;
-                ra[kk] = al;
-                kk++;
-              }
-            }
-          }
-          nr = kk;
-        }
+      } else {
+        nr = bilinear_roots(Bl, xl, td, n1, n2, rs, rt, ra);
+      }
+      if (kind == PT_FACE_CURVED && !clip_all) {
+        // the curved face lies within dev of its bilinear patch: a bilinear
+        // crossing far beyond the segment cannot refine into one inside it
+        const double dev = (double)__ldg(sl + 6);
+        const double reach = 4.0 * dev / fmax((double)fabsf(cosf_), 0.05) + 2.0 * k.band_x;
+        int kk = 0;
         #pragma unroll 1
         for (int i = 0; i < nr; ++i) {
-          double al = ra[i], s = rs[i], t = rt[i];
-          double mm = fmax(fabs(s), fabs(t));
-          if (mm > 1.0 + k.band_ref) continue;
-          if (al < a0 - k.band_x || al > L + k.band_x) continue;
-          if (fabs(mm - 1.0) < k.band_ref || fabs(al - a0) < k.band_x ||
-              fabs(L - al) < k.band_x) {
-            const int bcf = finfo_bc(info);
-            st |= PT_ST_NEAR_FACE |
-                  ((bcf == PT_BC_WALL || bcf == PT_BC_OPEN) ? (unsigned)PT_ST_NEAR_WALL : 0u);
-          }
-          if (mm <= 1.0 && al > a0 && al <= L && al < best) {
-            best = al;
-            bf = f;
-            bs = s;
-            bt = t;
+          double s = rs[i], t = rt[i], al = ra[i];
+          if (!(fabs(s) < 2.0 && fabs(t) < 2.0)) continue;
+          if (al > L + reach || al < a0 - reach) continue;
+          if (curved_refine<G>(X64, m.xg32 + (size_t)e * 3 * G * G * G, f, xl, td, k, s, t,
+                               al, L)) {
+            bool dup = false;
+            for (int j = 0; j < kk; ++j)
+              if (fabs(rs[j] - s) < 1e-10 && fabs(rt[j] - t) < 1e-10) dup = true;
+            if (!dup) {
+              rs[kk] = s;
+              rt[kk] = t;
+              ra[kk] = al;
+              kk++;
+            }
           }
         }
+        nr = kk;
       }
-    }
-    if (kFast && pf >= 0 && npro == 1 && !exact_seen) {
-      best = (double)pa32;
-      bf = pf;
-      bs = (double)ps32;
-      bt = (double)pt32;
+      #pragma unroll 1
+      for (int i = 0; i < nr; ++i) {
+        double al = ra[i], s = rs[i], t = rt[i];
+        double mm = fmax(fabs(s), fabs(t));
+        if (mm > 1.0 + k.band_ref) continue;
+        if (al < a0 - k.band_x || al > L + k.band_x) continue;
+        if (fabs(mm - 1.0) < k.band_ref || fabs(al - a0) < k.band_x ||
+            fabs(L - al) < k.band_x) {
+          const int bcf = finfo_bc(info);
+          st |= PT_ST_NEAR_FACE |
+                ((bcf == PT_BC_WALL || bcf == PT_BC_OPEN) ? (unsigned)PT_ST_NEAR_WALL : 0u);
+        }
+        if (mm <= 1.0 && al > a0 && al <= L && al < best) {
+          best = al;
+          bf = f;
+          bs = s;
+          bt = t;
+        }
+      }
     }
     if (bf < 0) break;
     const int info = __ldg(m.finfo + 6 * (size_t)e + bf);

@@ -44,6 +44,9 @@ struct DevMesh {
   const float* xg32;      // [E][3][g^3]   nodes - ce, FP32, coordinate-major
   const float* mono;      // [E][3][CS]    monomial coefficients of nodes - ce (pt_map.cuh),
   const float* monolo;    //               high and low FP32 parts
+  const float* curv;      // [E][4]        bounds on |second derivatives| of the three
+                          //               coordinates of the map for |xi| <= 1.1 (sum over
+                          //               a pair of directions; fourth word unused)
   const double* ce;       // [E][3]
   const float* tri;       // [E][12]       trilinear centre (3) and inverse Jacobian (9)
   const int* tmask;       // [E]           bit q: coordinate q is trilinear in xi (8-corner form)
@@ -68,6 +71,7 @@ struct DevConsts {
   float A32[5], B32[5];
   double mu, rho_p, g[3], mask[3];
   double newton_tol, band_ref, band_x, lost_tol;
+  float band_ref32, band_x32;
   double hl[4];                      // Haider-Levenspiel A, B, C, D
   int drag_law, max_newton, max_cross, guess, lift, track, buoyancy, curved_clip;
   double gbz[PT_MAXG * PT_MAXG];     // Bezier control values = gbz x nodal values
@@ -171,6 +175,9 @@ struct StageArgs {
   unsigned* list;         // [n] listed positions (| 1 << 31: walk only)
   unsigned* count;        // entries in list
   unsigned* count_next;   // the next stage's counter (cleared by this stage)
+  unsigned* list2;        // FP32 mode: [n] listed positions left to the FP64 intersection,
+  unsigned* count2;       //            their number, and the next stage's counter
+  unsigned* count2_next;
   int stage;              // 0..4
   double dt;
   unsigned long long* stats;
@@ -203,9 +210,10 @@ int max_active_push(int g, bool fp64, int np, int block);
 int launch_terms(int g, bool fp64, int np, const TermsArgs& a, int grid, int block, void* stream);
 // staged schedule: op 0 gather, 1 stage, 2 track, 3 learned start, 4 scatter back
 // (5, 6: the learned start of global positions a.x, tensor-core and warp-MMA
-// forms, for pt_mlp_start)
+// forms, for pt_mlp_start), 7 the FP64 intersections that the FP32 mode's track
+// leaves
 enum { PT_SOP_GATHER = 0, PT_SOP_STAGE = 1, PT_SOP_TRACK = 2, PT_SOP_GUESS = 3, PT_SOP_SCATTER = 4,
-       PT_SOP_GUESS_X_TC = 5, PT_SOP_GUESS_X_WARP = 6 };
+       PT_SOP_GUESS_X_TC = 5, PT_SOP_GUESS_X_WARP = 6, PT_SOP_EXACT = 7 };
 int launch_staged(int g, bool fp64, int np, int op, const StageArgs& a, const DevParticles& p,
                   const int* perm, int grid, int block, void* stream);
 int max_active_stage(int g, bool fp64, int np, int block);

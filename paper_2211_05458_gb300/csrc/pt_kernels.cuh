@@ -379,6 +379,7 @@ __device__ __noinline__ int settle_f32(const DevMesh& m, const DevConsts& k, int
       if (!newton_df<G>(m, k, e, xd, g, zd, it32, it64)) return 1;
     }
     have = false;
+    if (tmax3(zd[0].hi, zd[1].hi, zd[2].hi) < 1.f - 1e-5f) return 0;  // decided in FP32
     const double z[3] = {df_to_double(zd[0]), df_to_double(zd[1]), df_to_double(zd[2])};
     if (tmax3(z[0], z[1], z[2]) <= 1.0 + wtol) return 0;
     if (w == 4) return tmax3(z[0], z[1], z[2]) <= 1.0 + k.lost_tol ? 0 : 2;
@@ -608,7 +609,9 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
       if (!live) continue;
       df zd[3];
       int i32 = 0, i64 = 0;
-      bool ok = newton_df<G>(m, k, e, xd, guess, zd, i32, i64);
+      float Ji[9];
+      bool jok;
+      bool ok = newton_df<G>(m, k, e, xd, guess, zd, i32, i64, Ji, jok);
       c.it32 += i32;
       c.it64 += i64;
       if (!ok) {
@@ -637,6 +640,7 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
             live = false;
             continue;
           }
+          jok = false;  // Ji belongs to the element left
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
             xi[q] = zd[q].hi + zd[q].lo;
@@ -661,16 +665,20 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
       float acc[3];
       particle_accel_f32<G, NP>(m, k, U + (size_t)e * 5 * N3, e, zd, Uv, v, d, tau, st, acc);
       df xe[3];
-      float bf[3];
+      float dx[3];
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
         kx[r] = As * kx[r] + dt * v[r];
         kv[r] = As * kv[r] + dt * acc[r];
-        xe[r] = df_add(xd[r], df_from(Bs * kx[r]));
-        bf[r] = xe[r].hi;
+        dx[r] = Bs * kx[r];
+        xe[r] = df_add(xd[r], df_from(dx[r]));
         v[r] = v[r] + Bs * kv[r];
       }
-      const int touch = slab_touch(m, e, xf, bf);
+      int touch = 0;
+      if (!(jok && stays_inside(m, e, xi, Ji, dx, k.band_x32))) {
+        const float bf[3] = {xe[0].hi, xe[1].hi, xe[2].hi};
+        touch = slab_touch(m, e, xf, bf);
+      }
       if (!(touch & (k.track == PT_TRACK_REFERENCE ? 2 : 1))) {
         // no face reachable, or (localisation) no wall or open face: the end
         // point's owner is found by the next inverse map
@@ -678,27 +686,33 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
         for (int r = 0; r < 3; ++r) xd[r] = xe[r];
         if (touch) pending = true;
       } else {
-        // exact tracking in FP64 on global positions, then back to local
-        const double* ce = m.ce + 3 * (size_t)e;
-        double xs[3], xg[3];
+        int j32 = 0, j64 = 0;
+        const bool decided = track_f32<G>(m, k, e, xd, xe, st, j32, j64, c.tc);
+        c.it32 += j32;
+        c.it64 += j64;
+        if (!decided) {
+          // exact tracking in FP64 on global positions, then back to local
+          const double* ce = m.ce + 3 * (size_t)e;
+          double xs[3], xg[3];
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          const double cr = __ldg(ce + r);
-          xs[r] = cr + df_to_double(xd[r]);
-          xg[r] = cr + df_to_double(xe[r]);
+          for (int r = 0; r < 3; ++r) {
+            const double cr = __ldg(ce + r);
+            xs[r] = cr + df_to_double(xd[r]);
+            xg[r] = cr + df_to_double(xe[r]);
+          }
+          track_slow<G, float, CLIP>(m, k, e, xs, xg, v, kx, kv, hits, st, c.tc);
+          if (st & PT_ST_FROZEN) {
+            live = false;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) x[r] = xs[r];
+            moved = true;
+            continue;
+          }
+          const double* cn = m.ce + 3 * (size_t)e;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) xd[r] = df_from_double(xs[r] - __ldg(cn + r));
         }
-        track_slow<G, float, CLIP>(m, k, e, xs, xg, v, kx, kv, hits, st, c.tc);
-        if (st & PT_ST_FROZEN) {
-          live = false;
-#pragma unroll
-          for (int r = 0; r < 3; ++r) x[r] = xs[r];
-          moved = true;
-          continue;
-        }
-        const double* cn = m.ce + 3 * (size_t)e;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) xd[r] = df_from_double(xs[r] - __ldg(cn + r));
-        pending = true;
+        pending = !decided;
       }
     }
     if (live) ++c.steps;
@@ -1379,10 +1393,17 @@ struct Family {
           else
             k_track_f64<G, false><<<grid, block, 0, s>>>(a);
         } else {
+          k_track_f32<G><<<grid, 64, 0, s>>>(a);
+        }
+        break;
+      case PT_SOP_EXACT:
+        if constexpr (F64) {
+          return (int)cudaErrorInvalidValue;
+        } else {
           if (clip)
-            k_track_f32<G, true><<<grid, block, 0, s>>>(a);
+            k_exact_f32<G, true><<<grid, 32, 0, s>>>(a);
           else
-            k_track_f32<G, false><<<grid, block, 0, s>>>(a);
+            k_exact_f32<G, false><<<grid, 32, 0, s>>>(a);
         }
         break;
       case PT_SOP_GUESS:

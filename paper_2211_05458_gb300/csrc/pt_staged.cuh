@@ -11,10 +11,11 @@
 //               drag, RK update and the FP32 slab test; a particle whose stage
 //               segment may touch a face (~0.5 % at the 64^3 workload) is
 //               appended to a compacted list instead of being intersected;
-//   k_track_*   the listed particles on full warps: exact tracking through
-//               the faces (Secs. 3.2.3, 3.2.4, 2.4) and the walk that checks
-//               the new owner (the missed-crossing repair of the resident
-//               push, run at once instead of at the next stage's start);
+//   k_track_*   the listed particles on full warps: tracking through the
+//               faces (Secs. 3.2.3, 3.2.4, 2.4) and the walk that checks the new
+//               owner (the missed-crossing repair of the resident push, run at
+//               once instead of at the next stage's start); in FP32 mode the
+//               segments that need an FP64 intersection go on to k_exact_f32;
 // and, with the learned start, k_guess_mlp before k_stage_*.  Between stages
 // the particle state goes through HBM in element-sorted order: k_gather
 // copies it from the caller's arrays into library-owned structure-of-arrays
@@ -39,15 +40,17 @@ constexpr unsigned kSettleOnly = 0x80000000u;
 
 // Appends t (| flag) for every lane with want != 0; warp-collective (all 32
 // lanes must call it).
-__device__ __forceinline__ void list_append(const StageArgs& a, int64_t t, unsigned want) {
+__device__ __forceinline__ void list_append(unsigned* list, unsigned* count, int64_t t,
+                                            unsigned want) {
   const unsigned m = __ballot_sync(0xffffffffu, want != 0u);
   if (!m) return;
   const int lane = threadIdx.x & 31;
   const int leader = __ffs(m) - 1;
   unsigned base = 0u;
-  if (lane == leader) base = atomicAdd(a.count, (unsigned)__popc(m));
+  if (lane == leader) base = atomicAdd(count, (unsigned)__popc(m));
   base = __shfl_sync(0xffffffffu, base, leader);
-  if (want) a.list[base + __popc(m & ((1u << lane) - 1u))] = (unsigned)t | (want == 2u ? kSettleOnly : 0u);
+  if (want)
+    list[base + __popc(m & ((1u << lane) - 1u))] = (unsigned)t | (want == 2u ? kSettleOnly : 0u);
 }
 
 // Per-thread histogram of small counts: four 16-bit bins per word (a thread
@@ -168,7 +171,9 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
   }
   df zd[3];
   int i32 = 0, i64 = 0;
-  const bool ok = newton_df<G>(a.m, a.k, e, xd, guess, zd, i32, i64);
+  float Ji[9];
+  bool jok;
+  const bool ok = newton_df<G>(a.m, a.k, e, xd, guess, zd, i32, i64, Ji, jok);
   c.it32 += i32;
   c.it64 += i64;
   h32.add(i32);
@@ -198,16 +203,20 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
   particle_accel_f32<G, NP>(a.m, a.k, Ue, e, zd, Uv, v, d, tau, st, acc);
   const float As = a.k.A32[s], Bs = a.k.B32[s], dt = (float)a.dt;
   df xe[3];
-  float bf[3];
+  float dx[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     kx[r] = As * kx[r] + dt * v[r];
     kv[r] = As * kv[r] + dt * acc[r];
-    xe[r] = df_add(xd[r], df_from(Bs * kx[r]));
-    bf[r] = xe[r].hi;
+    dx[r] = Bs * kx[r];
+    xe[r] = df_add(xd[r], df_from(dx[r]));
     v[r] = v[r] + Bs * kv[r];
   }
-  const int touch = slab_touch(a.m, e, xf, bf);
+  int touch = 0;
+  if (!(jok && stays_inside(a.m, e, xi, Ji, dx, a.k.band_x32))) {
+    const float bf[3] = {xe[0].hi, xe[1].hi, xe[2].hi};
+    touch = slab_touch(a.m, e, xf, bf);
+  }
   unsigned list = 0u;
   if (!(touch & (a.k.track == PT_TRACK_REFERENCE ? 2 : 1))) {
     // no face reachable, or (localisation) no wall or open face: with a touch
@@ -241,7 +250,7 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
 
 template <int G, int NP, bool MLP>
 __global__ void __launch_bounds__(128, PT_STAGE_MINB) k_stage_f32(const __grid_constant__ StageArgs a) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_next = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_next = *a.count2_next = 0u;
   PushCounters c = {0, 0, 0, {0, 0, 0}};
   Hist8 h32, h64;
   const int64_t n = a.n;
@@ -254,65 +263,120 @@ __global__ void __launch_bounds__(128, PT_STAGE_MINB) k_stage_f32(const __grid_c
     StageIn in;
     if (t < n) stage_load<MLP>(a, t, in);
     const unsigned want = t < n ? stage_one_f32<G, NP, MLP>(a, t, in, c, h32, h64, sb) : 0u;
-    list_append(a, t, want);
+    list_append(a.list, a.count, t, want);
   }
   stage_counters(a, c);
   h32.flush(a.stats, PT_C_H32, 8);
   h64.flush(a.stats, PT_C_H64, 8);
 }
 
-// Exact tracking of the listed stage segments, then the walk that checks the
-// new owner; FP64 on global positions, back to the double-float offset.
-#ifndef PT_TRACK_MINB
-#define PT_TRACK_MINB 1
-#endif
+// The listed stage segments, first pass: tracking in reference space (track_f32)
+// or the walk.  Segments that it does not decide (walls, open and mortar faces,
+// ends and edges within the bands) go to a second list for k_exact_f32, so that
+// no warp of this pass waits for an FP64 intersection.  Both passes are
+// latency-bound (about a thousand segments per stage and 10^6 particles): 64
+// threads per block spread them over the SMs.
+template <int G>
+__global__ void __launch_bounds__(64, 4) k_track_f32(const __grid_constant__ StageArgs a) {
+  PushCounters c = {0, 0, 0, {0, 0, 0}};
+  Hist8 hcr;
+  const int64_t n = a.n;
+  const unsigned cnt = *a.count;
+  const float* xeg = reinterpret_cast<const float*>(a.xe);
+  const unsigned stride = gridDim.x * blockDim.x;
+  const unsigned cround = (cnt + 31u) & ~31u;  // whole warps
+  if (((blockIdx.x * blockDim.x + threadIdx.x) & ~31u) >= cround) return;
+  for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < cround; j += stride) {
+    unsigned exact = 0u, t32 = 0u;
+    if (j < cnt) {
+      const unsigned ent = a.list[j];
+      t32 = ent & ~kSettleOnly;
+      const int64_t t = t32;
+      int e = a.e[t];
+      const int e0 = e;
+      df xd[3];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) xd[r] = df{a.xh[r * n + t], a.xl[r * n + t]};
+      int cr = 0, j32 = 0, j64 = 0, rc = 0;
+      if (!(ent & kSettleOnly)) {
+        df xe[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) xe[r] = df{xeg[r * n + t], xeg[(3 + r) * n + t]};
+        const int cr0 = c.tc.cross;
+        unsigned bits = 0u;
+        exact = track_f32<G>(a.m, a.k, e, xd, xe, bits, j32, j64, c.tc) ? 0u : 1u;
+        if (!exact) hcr.add(c.tc.cross - cr0);
+        if (bits) a.st[t] |= bits;
+      } else {
+        df zd[3];
+        rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr);
+      }
+      c.it32 += j32;
+      c.it64 += j64;
+      if (!exact) {
+        c.tc.cross += cr;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          a.xh[r * n + t] = xd[r].hi;
+          a.xl[r * n + t] = xd[r].lo;
+        }
+        if (e != e0) a.e[t] = e;
+        if (rc)
+          a.st[t] |= rc == 1 ? PT_ST_NEWTON_FAIL : PT_ST_LOST;
+        else if (a.stage == 4)
+          ++c.steps;
+      }
+    }
+    list_append(a.list2, a.count2, t32, exact);
+  }
+  stage_counters(a, c);
+  hcr.flush(a.stats, PT_C_HCR, 4);
+}
+
+// Second pass: the FP64 intersection of the segments the first pass left, on
+// global positions, back to the double-float offset, and the walk.  One FP64
+// instruction holds an SM's FP64 unit for the same time whether one lane or 32
+// are active and these lanes rarely agree on a path, so the entries are spread
+// over all warps of the grid, one per warp while there are that few.
 template <int G, bool CLIP>
-__global__ void __launch_bounds__(128, PT_TRACK_MINB) k_track_f32(const __grid_constant__ StageArgs a) {
+__global__ void __launch_bounds__(32) k_exact_f32(const __grid_constant__ StageArgs a) {
   PushCounters c = {0, 0, 0, {0, 0, 0}};
   Hist8 hcr;
   const int64_t n = a.n;
   const int s = a.stage;
-  const unsigned cnt = *a.count;
+  const unsigned cnt = *a.count2;
+  if (blockIdx.x >= cnt) return;
   float* vg = reinterpret_cast<float*>(a.v);
   float* kxg = reinterpret_cast<float*>(a.kx);
   float* kvg = reinterpret_cast<float*>(a.kv);
   const float* xeg = reinterpret_cast<const float*>(a.xe);
   const unsigned stride = gridDim.x * blockDim.x;
-  const unsigned cround = (cnt + stride - 1) / stride * stride;
-  for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < cround; j += stride) {
-    if (j >= cnt) continue;
-    const unsigned ent = a.list[j];
-    const int64_t t = ent & ~kSettleOnly;
+  // entry j of warp w is w + j gridDim
+  for (unsigned j = blockIdx.x + gridDim.x * threadIdx.x; j < cnt; j += stride) {
+    const int64_t t = a.list2[j];
     unsigned st = a.st[t];
     int e = a.e[t], hits = a.hits[t];
     df xd[3];
     float v[3], kx[3], kv[3];
+    double xs[3], xg[3];
+    const double* ce = a.m.ce + 3 * (size_t)e;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       xd[r] = df{a.xh[r * n + t], a.xl[r * n + t]};
       v[r] = vg[r * n + t];
       kx[r] = kxg[r * n + t];  // stale at the last stage of a step: not used after it
       kv[r] = kvg[r * n + t];
+      const double cr = __ldg(ce + r);
+      xs[r] = cr + df_to_double(xd[r]);
+      xg[r] = cr + df_to_double(df{xeg[r * n + t], xeg[(3 + r) * n + t]});
     }
-    bool frozen = false;
-    if (!(ent & kSettleOnly)) {
-      const double* ce = a.m.ce + 3 * (size_t)e;
-      double xs[3], xg[3];
+    const int cr0 = c.tc.cross;
+    track_slow<G, float, CLIP>(a.m, a.k, e, xs, xg, v, kx, kv, hits, st, c.tc);
+    hcr.add(c.tc.cross - cr0);
+    const double* cn = a.m.ce + 3 * (size_t)e;
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const double cr = __ldg(ce + r);
-        xs[r] = cr + df_to_double(xd[r]);
-        xg[r] = cr + df_to_double(df{xeg[r * n + t], xeg[(3 + r) * n + t]});
-      }
-      const int cr0 = c.tc.cross;
-      track_slow<G, float, CLIP>(a.m, a.k, e, xs, xg, v, kx, kv, hits, st, c.tc);
-      hcr.add(c.tc.cross - cr0);
-      const double* cn = a.m.ce + 3 * (size_t)e;
-#pragma unroll
-      for (int r = 0; r < 3; ++r) xd[r] = df_from_double(xs[r] - __ldg(cn + r));
-      frozen = (st & PT_ST_FROZEN) != 0;
-    }
-    if (!frozen) {
+    for (int r = 0; r < 3; ++r) xd[r] = df_from_double(xs[r] - __ldg(cn + r));
+    if (!(st & PT_ST_FROZEN)) {
       df zd[3];
       int cr = 0, j32 = 0, j64 = 0;
       const int rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr);
@@ -336,6 +400,7 @@ __global__ void __launch_bounds__(128, PT_TRACK_MINB) k_track_f32(const __grid_c
     a.st[t] = st;
     if (s == 4 && !(st & PT_ST_FROZEN)) ++c.steps;
   }
+  __syncwarp();
   stage_counters(a, c);
   hcr.flush(a.stats, PT_C_HCR, 4);
 }
@@ -559,7 +624,7 @@ __device__ __forceinline__ unsigned stage_one_f64(const StageArgs& a, int64_t t,
 
 template <int G, int NP>
 __global__ void __launch_bounds__(128, PT_PUSH_MINB_F64) k_stage_f64(const __grid_constant__ StageArgs a) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_next = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_next = *a.count2_next = 0u;
   PushCounters c = {0, 0, 0, {0, 0, 0}};
   Hist8 h64;
   const int64_t n = a.n;
@@ -567,7 +632,7 @@ __global__ void __launch_bounds__(128, PT_PUSH_MINB_F64) k_stage_f64(const __gri
   const int64_t nround = (n + stride - 1) / stride * stride;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nround; t += stride) {
     const unsigned want = t < n ? stage_one_f64<G, NP>(a, t, c, h64) : 0u;
-    list_append(a, t, want);
+    list_append(a.list, a.count, t, want);
   }
   stage_counters(a, c);
   h64.flush(a.stats, PT_C_H64, 8);
