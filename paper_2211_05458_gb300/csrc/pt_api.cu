@@ -765,6 +765,14 @@ static void fill_consts(const pt_ctx* c, DevConsts& k) {
     k.hl[2] = std::exp(4.905 - 13.8944 * f + 18.4222 * f * f - 10.2599 * f * f * f);
     k.hl[3] = std::exp(1.4681 + 12.2584 * f - 20.7322 * f * f + 15.8855 * f * f * f);
   }
+  k.mu32 = (float)k.mu;
+  k.rho_p32 = (float)k.rho_p;
+  k.newton_tol32 = (float)k.newton_tol;
+  for (int r = 0; r < 3; ++r) {
+    k.g32[r] = (float)k.g[r];
+    k.mask32[r] = (float)k.mask[r];
+  }
+  for (int q = 0; q < 4; ++q) k.hl32[q] = (float)k.hl[q];
   k.max_newton = c->cfg.max_newton;
   k.max_cross = c->cfg.max_cross;
   k.guess = c->cfg.guess;
@@ -1117,6 +1125,7 @@ static pt_status staged_prepare(pt_ctx* c, const pt_particles* p, double dt, Sta
   a.U = c->U;
   a.n = n;
   a.dt = dt;
+  a.dt32 = (float)dt;
   a.stats = c->d_stats;
   L.dp = {n, p->x, p->v, p->d, p->elem, p->hits, p->status};
   const int occ = max_active_stage(c->g, L.f64, L.np, L.block);

@@ -66,6 +66,27 @@ struct Nodes<double> {
   __device__ static const double* solw(const DevConsts& k) { return k.sw; }
 };
 
+// physical constants of the right precision (a conversion from FP64 inside a
+// kernel would hold an SM's FP64 unit for 64 cycles per warp)
+template <typename T>
+struct Phys;
+template <>
+struct Phys<float> {
+  __device__ static float mu(const DevConsts& k) { return k.mu32; }
+  __device__ static float rho_p(const DevConsts& k) { return k.rho_p32; }
+  __device__ static const float* g(const DevConsts& k) { return k.g32; }
+  __device__ static const float* mask(const DevConsts& k) { return k.mask32; }
+  __device__ static const float* hl(const DevConsts& k) { return k.hl32; }
+};
+template <>
+struct Phys<double> {
+  __device__ static double mu(const DevConsts& k) { return k.mu; }
+  __device__ static double rho_p(const DevConsts& k) { return k.rho_p; }
+  __device__ static const double* g(const DevConsts& k) { return k.g; }
+  __device__ static const double* mask(const DevConsts& k) { return k.mask; }
+  __device__ static const double* hl(const DevConsts& k) { return k.hl; }
+};
+
 // Lagrange basis in barycentric product form: l_i(x) = w_i prod_{m != i} (x - x_m),
 // w_i = 1 / prod_{m != i} (x_i - x_m).  Prefix and suffix products avoid the
 // division of the second barycentric form, so the values at the nodes are exact.
@@ -274,7 +295,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
   if (have) {
 #pragma unroll
     for (int q = 0; q < 3; ++q) zd[q] = df_from(z[q]);
-    const float tol = (float)k.newton_tol;
+    const float tol = k.newton_tol32;
     // Each step needs the residual at the current iterate.  The first is the
     // double-float residual at the FP32 iterate z.  After a first step d with
     // |d| <= 4e-7 the next residual is r(z) + [chi(z - d) - chi(z)], and the
@@ -357,108 +378,143 @@ __device__ __forceinline__ bool newton_mixed(const DevMesh& m, const DevConsts& 
 // interpolation of rho and rho u (Eq. part_interpolation), sum-factorised
 // ---------------------------------------------------------------------------
 
-// FP32 at N = 5 takes two variables per pass (their row loads independent:
-// twice the loads in flight; +5 % at the 64^3 workload).  SS > 0: the
-// third-direction basis and the results, indexed by the rolled loops, go
-// through this thread's column of a [kScratchRows][SS] shared array at sb
-// instead of through local memory.
-constexpr int kScratchRows = 12;
-template <int NP, typename T, int SS = 0>
-__device__ __forceinline__ void interp4(const T* __restrict__ Ue, const T* l1, const T* l2,
-                                        const T* l3, T* out, float* sb = nullptr) {
-  constexpr int N3 = NP * NP * NP;
-  // two variables per pass: their row loads are independent, which doubles
-  // the loads in flight per iteration
-  if constexpr (std::is_same<T, float>::value && NP == 6) {
-    // rows kk: l3; NP + v: the results
-    constexpr bool kS = SS > 0;
-    if constexpr (kS) {
+// FP32, sum-factorised, the sum over a row in packed pairs (its even and odd
+// nodes, joined at the end).  NP = 6 takes two variables per pass: twice the
+// loads in flight, which is what the staged push is short of (weights of a whole
+// plane in registers save another 150 instructions per particle, but leave
+// room for fewer loads: 312 against 235 us per stage of 10^6 particles).  The
+// third-direction basis is shifted through registers by the rolled loop, which
+// keeps it out of local memory.
+template <int NP>
+__device__ __forceinline__ void interp4(const float* __restrict__ Ue, const float* l1,
+                                        const float* l2, const float* l3, float* out) {
+  constexpr int N2 = NP * NP, N3 = N2 * NP, NH = NP / 2;
+  if constexpr (NP % 2 == 0) {
+    constexpr int VB = NP == 6 ? 2 : 1;  // variables per pass
+    f32x2 w1[NH];
 #pragma unroll
-      for (int kk = 0; kk < NP; ++kk) sb[kk * SS] = l3[kk];
-    }
+    for (int i = 0; i < NH; ++i) w1[i] = pk2(l1[2 * i], l1[2 * i + 1]);
+    float lk[NP], res[4];
+#pragma unroll
+    for (int c = 0; c < NP; ++c) lk[c] = l3[c];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) res[v] = 0.f;
 #pragma unroll 1
-    for (int v = 0; v < 4; v += 2) {
-      const float* Ua = Ue + v * N3;
-      const float* Ub = Ua + N3;
-      float acca = 0.f, accb = 0.f;
+    for (int v = 0; v < 4; v += VB) {
+      f32x2 acc[VB];
+#pragma unroll
+      for (int q = 0; q < VB; ++q) acc[q] = dup2(0.f);
 #pragma unroll 1
       for (int kk = 0; kk < NP; ++kk) {
-        float ta = 0.f, tb = 0.f;
+        const f32x2 lz = dup2(lk[0]);
+        {  // rotate: after NP iterations the basis is in place again
+          const float l0 = lk[0];
 #pragma unroll
-        for (int j = 0; j < NP; j += 2) {
-          const float4* qa = reinterpret_cast<const float4*>(Ua + NP * (j + NP * kk));
-          const float4* qb = reinterpret_cast<const float4*>(Ub + NP * (j + NP * kk));
-          const float4 a0 = __ldg(qa), a1 = __ldg(qa + 1), a2 = __ldg(qa + 2);
-          const float4 b0 = __ldg(qb), b1 = __ldg(qb + 1), b2 = __ldg(qb + 2);
-          const float ra0[6] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y};
-          const float ra1[6] = {a1.z, a1.w, a2.x, a2.y, a2.z, a2.w};
-          const float rb0[6] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y};
-          const float rb1[6] = {b1.z, b1.w, b2.x, b2.y, b2.z, b2.w};
-          float sa0 = 0.f, sa1 = 0.f, sb0 = 0.f, sb1 = 0.f;
+          for (int c = 0; c + 1 < NP; ++c) lk[c] = lk[c + 1];
+          lk[NP - 1] = l0;
+        }
+        f32x2 u[VB][N2 / 2];
+#pragma unroll
+        for (int q = 0; q < VB; ++q) {
+          const ulonglong2* P =
+              reinterpret_cast<const ulonglong2*>(Ue + (v + q) * N3 + kk * N2);
+#pragma unroll
+          for (int i = 0; i < N2 / 4; ++i) {
+            const ulonglong2 x = __ldg(P + i);
+            u[q][2 * i] = x.x;
+            u[q][2 * i + 1] = x.y;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < VB; ++q) {
+          f32x2 t;
+#pragma unroll
+          for (int j = 0; j < NP; ++j) {
+            f32x2 t1 = mul2(u[q][j * NH], w1[0]);
+#pragma unroll
+            for (int i = 1; i < NH; ++i) t1 = fma2(u[q][j * NH + i], w1[i], t1);
+            t = j ? fma2(t1, dup2(l2[j]), t) : mul2(t1, dup2(l2[0]));
+          }
+          acc[q] = fma2(t, lz, acc[q]);
+        }
+      }
+      // the results move up the registers (v is a run-time index)
+#pragma unroll
+      for (int q = 0; q + VB < 4; ++q) res[q] = res[q + VB];
+#pragma unroll
+      for (int q = 0; q < VB; ++q) {
+        float x, y;
+        unpk2(acc[q], x, y);
+        res[4 - VB + q] = x + y;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) out[v] = res[v];
+  } else {
+    float lk[NP], res[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < NP; ++c) lk[c] = l3[c];
+    f32x2 w2[NP];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) w2[j] = dup2(l2[j]);
+    // single values are read (rows of odd length have no alignment): two
+    // variables per packed operation instead
+#pragma unroll 1
+    for (int v = 0; v < 4; v += 2) {
+      f32x2 acc = dup2(0.f);
+#pragma unroll 1
+      for (int kk = 0; kk < NP; ++kk) {
+        const f32x2 lz = dup2(lk[0]);
+        {
+          const float l0 = lk[0];
+#pragma unroll
+          for (int c = 0; c + 1 < NP; ++c) lk[c] = lk[c + 1];
+          lk[NP - 1] = l0;
+        }
+        const float* P = Ue + v * N3 + kk * N2;
+        f32x2 t;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          f32x2 t1;
 #pragma unroll
           for (int i = 0; i < NP; ++i) {
-            sa0 = fmaf(ra0[i], l1[i], sa0);
-            sa1 = fmaf(ra1[i], l1[i], sa1);
-            sb0 = fmaf(rb0[i], l1[i], sb0);
-            sb1 = fmaf(rb1[i], l1[i], sb1);
+            const f32x2 x = pk2(__ldg(P + j * NP + i), __ldg(P + N3 + j * NP + i));
+            t1 = i ? fma2(x, dup2(l1[i]), t1) : mul2(x, dup2(l1[0]));
           }
-          ta = fmaf(sa0, l2[j], ta);
-          ta = fmaf(sa1, l2[j + 1], ta);
-          tb = fmaf(sb0, l2[j], tb);
-          tb = fmaf(sb1, l2[j + 1], tb);
+          t = j ? fma2(t1, w2[j], t) : mul2(t1, w2[0]);
         }
-        const float lk = kS ? sb[kk * SS] : l3[kk];
-        acca = fmaf(ta, lk, acca);
-        accb = fmaf(tb, lk, accb);
+        acc = fma2(t, lz, acc);
       }
-      if constexpr (kS) {
-        sb[(NP + v) * SS] = acca;
-        sb[(NP + 1 + v) * SS] = accb;
-      } else {
-        out[v] = acca;
-        out[v + 1] = accb;
-      }
+      res[0] = res[2];
+      res[1] = res[3];
+      unpk2(acc, res[2], res[3]);
     }
-    if constexpr (kS) {
 #pragma unroll
-      for (int v = 0; v < 4; ++v) out[v] = sb[(NP + v) * SS];
-    }
-    return;
+    for (int v = 0; v < 4; ++v) out[v] = res[v];
   }
+}
+
+// FP64: sum-factorised
+template <int NP>
+__device__ __forceinline__ void interp4(const double* __restrict__ Ue, const double* l1,
+                                        const double* l2, const double* l3, double* out) {
+  constexpr int N3 = NP * NP * NP;
 #pragma unroll 1
   for (int v = 0; v < 4; ++v) {
-    const T* Uv = Ue + v * N3;
-    T acc = T(0);
+    const double* Uv = Ue + v * N3;
+    double acc = 0.0;
 #pragma unroll 1
     for (int kk = 0; kk < NP; ++kk) {
-      T t2 = T(0);
+      double t2 = 0.0;
 #pragma unroll
       for (int j = 0; j < NP; ++j) {
-        const T* row = Uv + NP * (j + NP * kk);
-        T t1 = T(0);
-        if constexpr (std::is_same<T, float>::value && NP % 4 == 0) {
+        const double* row = Uv + NP * (j + NP * kk);
+        double t1 = 0.0;
 #pragma unroll
-          for (int i = 0; i < NP; i += 4) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(row + i));
-            t1 = tfma((T)q.x, l1[i], t1);
-            t1 = tfma((T)q.y, l1[i + 1], t1);
-            t1 = tfma((T)q.z, l1[i + 2], t1);
-            t1 = tfma((T)q.w, l1[i + 3], t1);
-          }
-        } else if constexpr (std::is_same<T, float>::value && NP % 2 == 0) {
-#pragma unroll
-          for (int i = 0; i < NP; i += 2) {
-            const float2 q = __ldg(reinterpret_cast<const float2*>(row + i));
-            t1 = tfma((T)q.x, l1[i], t1);
-            t1 = tfma((T)q.y, l1[i + 1], t1);
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) t1 = tfma(__ldg(row + i), l1[i], t1);
-        }
-        t2 = tfma(t1, l2[j], t2);
+        for (int i = 0; i < NP; ++i) t1 = fma(__ldg(row + i), l1[i], t1);
+        t2 = fma(t1, l2[j], t2);
       }
-      acc = tfma(t2, l3[kk], acc);
+      acc = fma(t2, l3[kk], acc);
     }
     out[v] = acc;
   }
@@ -475,8 +531,8 @@ template <typename T>
 __device__ __forceinline__ T drag_factor(const DevConsts& k, T re) {
   if (k.drag_law == 1) return T(1) + T(0.15) * tpow(re, T(0.687));
   if (!(re > T(0))) return T(1);
-  return T(1) + (T)k.hl[0] * tpow(re, (T)k.hl[1]) +
-         re / T(24) * (T)k.hl[2] / (T(1) + (T)k.hl[3] / re);
+  const T* h = Phys<T>::hl(k);
+  return T(1) + h[0] * tpow(re, h[1]) + re / T(24) * h[2] / (T(1) + h[3] / re);
 }
 
 // ---------------------------------------------------------------------------

@@ -71,7 +71,8 @@ struct DevConsts {
   float A32[5], B32[5];
   double mu, rho_p, g[3], mask[3];
   double newton_tol, band_ref, band_x, lost_tol;
-  float band_ref32, band_x32;
+  // FP32 copies for the FP32 mode's kernels
+  float mu32, rho_p32, g32[3], mask32[3], newton_tol32, band_ref32, band_x32, hl32[4];
   double hl[4];                      // Haider-Levenspiel A, B, C, D
   int drag_law, max_newton, max_cross, guess, lift, track, buoyancy, curved_clip;
   double gbz[PT_MAXG * PT_MAXG];     // Bezier control values = gbz x nodal values
@@ -180,6 +181,7 @@ struct StageArgs {
   unsigned* count2_next;
   int stage;              // 0..4
   double dt;
+  float dt32;
   unsigned long long* stats;
 };
 

@@ -231,7 +231,8 @@ __device__ __forceinline__ void particle_accel(const DevMesh& m, const DevConsts
                                                const R* __restrict__ Ue, int e, const double* xi,
                                                const R* Uv, const R* v, R d, R tau, unsigned& st,
                                                R* acc) {
-  const R mu = (R)k.mu;
+  const R mu = Phys<R>::mu(k);
+  const R *g = Phys<R>::g(k), *mask = Phys<R>::mask(k);
   R irho = R(1) / Uv[0], rel[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) rel[r] = Uv[1 + r] * irho - v[r];
@@ -245,13 +246,13 @@ __device__ __forceinline__ void particle_accel(const DevMesh& m, const DevConsts
   R al[3] = {R(0), R(0), R(0)};
   if (k.lift) {
     saffman_force<G, NP, R>(m, k, Ue, e, xi, v, d, al);
-    const R imp = R(6) / (R(3.14159265358979323846) * (R)k.rho_p * d * d * d);
+    const R imp = R(6) / (R(3.14159265358979323846) * Phys<R>::rho_p(k) * d * d * d);
 #pragma unroll
     for (int r = 0; r < 3; ++r) al[r] *= imp;
   }
-  const R gf = k.buoyancy ? R(1) - Uv[0] / (R)k.rho_p : R(1);
+  const R gf = k.buoyancy ? R(1) - Uv[0] / Phys<R>::rho_p(k) : R(1);
 #pragma unroll
-  for (int r = 0; r < 3; ++r) acc[r] = (R)k.mask[r] * coef * rel[r] + (R)k.g[r] * gf + al[r];
+  for (int r = 0; r < 3; ++r) acc[r] = mask[r] * coef * rel[r] + g[r] * gf + al[r];
 }
 
 // FP32 mode: as particle_accel, xi as a double-float (used by the lift only)
@@ -260,7 +261,7 @@ __device__ __forceinline__ void particle_accel_f32(const DevMesh& m, const DevCo
                                                    const float* __restrict__ Ue, int e,
                                                    const df* zd, const float* Uv, const float* v,
                                                    float d, float tau, unsigned& st, float* acc) {
-  const float mu = (float)k.mu;
+  const float mu = k.mu32;
   float irho = 1.f / Uv[0], rel[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) rel[r] = Uv[1 + r] * irho - v[r];
@@ -275,14 +276,14 @@ __device__ __forceinline__ void particle_accel_f32(const DevMesh& m, const DevCo
   if (k.lift) {
     const double xid[3] = {df_to_double(zd[0]), df_to_double(zd[1]), df_to_double(zd[2])};
     saffman_force<G, NP, float>(m, k, Ue, e, xid, v, d, al);
-    const float imp = 6.f / (3.14159265358979323846f * (float)k.rho_p * d * d * d);
+    const float imp = 6.f / (3.14159265358979323846f * k.rho_p32 * d * d * d);
 #pragma unroll
     for (int r = 0; r < 3; ++r) al[r] *= imp;
   }
-  const float gf = k.buoyancy ? 1.f - Uv[0] / (float)k.rho_p : 1.f;
+  const float gf = k.buoyancy ? 1.f - Uv[0] / k.rho_p32 : 1.f;
 #pragma unroll
   for (int r = 0; r < 3; ++r)
-    acc[r] = (float)k.mask[r] * coef * rel[r] + (float)k.g[r] * gf + al[r];
+    acc[r] = k.mask32[r] * coef * rel[r] + k.g32[r] * gf + al[r];
 }
 
 struct PushCounters {
@@ -500,7 +501,7 @@ __device__ __forceinline__ void push_particle(const DevMesh& m, const DevConsts&
       lagr<NP, R>((R)xi[0], Nodes<R>::sol(k), Nodes<R>::solw(k), l1);
       lagr<NP, R>((R)xi[1], Nodes<R>::sol(k), Nodes<R>::solw(k), l2);
       lagr<NP, R>((R)xi[2], Nodes<R>::sol(k), Nodes<R>::solw(k), l3);
-      interp4<NP, R>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
+      interp4<NP>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
       // drag + gravity
       R acc[3];
       particle_accel<G, NP, R>(m, k, U + (size_t)e * 5 * N3, e, xi, Uv, v, d, tau, st, acc);
@@ -564,7 +565,6 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
   constexpr int N3 = NP * NP * NP;
   const int64_t n = p.n;
   const float dt = (float)dtd;
-  const float mu = (float)k.mu;
   float* vg = reinterpret_cast<float*>(p.v);
   const float* dg = reinterpret_cast<const float*>(p.d);
   unsigned st = inrange ? p.status[ip] : PT_ST_FROZEN;
@@ -596,7 +596,7 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
   }
   bool moved = false;
   bool pending = false;  // the last stage took the exact tracking path
-  const float tau = (float)k.rho_p * d * d / (18.f * mu);
+  const float tau = k.rho_p32 * d * d / (18.f * k.mu32);
   for (int step = 0; step < nsteps; ++step) {
     float kx[3] = {0, 0, 0}, kv[3] = {0, 0, 0};
     for (int s = 0; s < 5; ++s) {
@@ -621,7 +621,7 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
       }
       float xi[3] = {zd[0].hi + zd[0].lo, zd[1].hi + zd[1].lo, zd[2].hi + zd[2].lo};
       const float mx = tmax3(xi[0], xi[1], xi[2]);
-      if (mx > 1.f - fmaxf(1e-5f, (float)k.band_ref)) {  // decide the bands exactly (rare)
+      if (mx > 1.f - fmaxf(1e-5f, k.band_ref32)) {  // decide the bands exactly (rare)
         double md = fmax(fmax(fabs(df_to_double(zd[0])), fabs(df_to_double(zd[1]))),
                          fabs(df_to_double(zd[2])));
         if (md > 1.0 + k.lost_tol && !pending) {  // outside without having moved: lost
@@ -660,7 +660,7 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
       lagr<NP, float>(xi[0], k.sn32, k.sw32, l1);
       lagr<NP, float>(xi[1], k.sn32, k.sw32, l2);
       lagr<NP, float>(xi[2], k.sn32, k.sw32, l3);
-      interp4<NP, float>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
+      interp4<NP>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
       // drag + gravity
       float acc[3];
       particle_accel_f32<G, NP>(m, k, U + (size_t)e * 5 * N3, e, zd, Uv, v, d, tau, st, acc);
@@ -911,8 +911,8 @@ __device__ __forceinline__ bool particle_source(const DepositArgs& a, int64_t ip
   lagr<NP, R>((R)xi[0], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), lr1);
   lagr<NP, R>((R)xi[1], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), lr2);
   lagr<NP, R>((R)xi[2], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), lr3);
-  interp4<NP, R>(reinterpret_cast<const R*>(a.U) + (size_t)e * 5 * N3, lr1, lr2, lr3, Uv);
-  const R mu = (R)a.k.mu;
+  interp4<NP>(reinterpret_cast<const R*>(a.U) + (size_t)e * 5 * N3, lr1, lr2, lr3, Uv);
+  const R mu = Phys<R>::mu(a.k);
   R rel[3];
   R irho = R(1) / Uv[0];
 #pragma unroll
@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(128) k_terms(const __grid_constant__ TermsArgs
       lagr<NP, R>((R)xi[0], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), l1);
       lagr<NP, R>((R)xi[1], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), l2);
       lagr<NP, R>((R)xi[2], Nodes<R>::sol(a.k), Nodes<R>::solw(a.k), l3);
-      interp4<NP, R>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
+      interp4<NP>(U + (size_t)e * 5 * N3, l1, l2, l3, Uv);
       particle_accel<G, NP, R>(a.m, a.k, U + (size_t)e * 5 * N3, e, xi, Uv, v, d, tau, st, acc);
     } else {
       df xd[3], zd[3];
@@ -1234,7 +1234,7 @@ __global__ void __launch_bounds__(128) k_terms(const __grid_constant__ TermsArgs
       lagr<NP, float>(xs[0], a.k.sn32, a.k.sw32, l1);
       lagr<NP, float>(xs[1], a.k.sn32, a.k.sw32, l2);
       lagr<NP, float>(xs[2], a.k.sn32, a.k.sw32, l3);
-      interp4<NP, float>(reinterpret_cast<const float*>(U) + (size_t)e * 5 * N3, l1, l2, l3,
+      interp4<NP>(reinterpret_cast<const float*>(U) + (size_t)e * 5 * N3, l1, l2, l3,
                          reinterpret_cast<float*>(Uv));
       particle_accel_f32<G, NP>(a.m, a.k, reinterpret_cast<const float*>(U) + (size_t)e * 5 * N3,
                                 e, zd, reinterpret_cast<const float*>(Uv),

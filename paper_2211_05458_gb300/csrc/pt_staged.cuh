@@ -134,11 +134,11 @@ __device__ __forceinline__ void stage_load(const StageArgs& a, int64_t t, StageI
 }
 
 // Returns 0 (stage end committed), 1 (listed for exact tracking) or 2 (listed
-// for the walk only).  sb: this thread's column of the interpolation's scratch.
+// for the walk only).
 template <int G, int NP, bool MLP>
 __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
                                                   const StageIn& in, PushCounters& c, Hist8& h32,
-                                                  Hist8& h64, float* sb) {
+                                                  Hist8& h64) {
   constexpr int N3 = NP * NP * NP;
   const int64_t n = a.n;
   const int s = a.stage;
@@ -159,8 +159,7 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
     kx[r] = in.kx[r];
     kv[r] = in.kv[r];
   }
-  const float mu = (float)a.k.mu;
-  const float tau = (float)a.k.rho_p * d * d / (18.f * mu);
+  const float tau = a.k.rho_p32 * d * d / (18.f * a.k.mu32);
   float xf[3] = {xd[0].hi, xd[1].hi, xd[2].hi};
   float guess[3];
   if constexpr (MLP) {
@@ -184,7 +183,7 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
   }
   const float xi[3] = {zd[0].hi + zd[0].lo, zd[1].hi + zd[1].lo, zd[2].hi + zd[2].lo};
   const float mx = tmax3(xi[0], xi[1], xi[2]);
-  if (mx > 1.f - fmaxf(1e-5f, (float)a.k.band_ref)) {  // decide the bands exactly (rare)
+  if (mx > 1.f - fmaxf(1e-5f, a.k.band_ref32)) {  // decide the bands exactly (rare)
     const double z[3] = {df_to_double(zd[0]), df_to_double(zd[1]), df_to_double(zd[2])};
     const double md = tmax3(z[0], z[1], z[2]);
     if (md > 1.0 + a.k.lost_tol) {  // outside: the walk after the last crossing ran already
@@ -199,9 +198,9 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
   lagr<NP, float>(xi[0], a.k.sn32, a.k.sw32, l1);
   lagr<NP, float>(xi[1], a.k.sn32, a.k.sw32, l2);
   lagr<NP, float>(xi[2], a.k.sn32, a.k.sw32, l3);
-  interp4<NP, float, 128>(Ue, l1, l2, l3, Uv, sb);
+  interp4<NP>(Ue, l1, l2, l3, Uv);
   particle_accel_f32<G, NP>(a.m, a.k, Ue, e, zd, Uv, v, d, tau, st, acc);
-  const float As = a.k.A32[s], Bs = a.k.B32[s], dt = (float)a.dt;
+  const float As = a.k.A32[s], Bs = a.k.B32[s], dt = a.dt32;
   df xe[3];
   float dx[3];
 #pragma unroll
@@ -256,13 +255,10 @@ __global__ void __launch_bounds__(128, PT_STAGE_MINB) k_stage_f32(const __grid_c
   const int64_t n = a.n;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t nround = (n + stride - 1) / stride * stride;  // uniform trip count per warp
-  // this thread's column of the interpolation's scratch (blocks of 128 threads)
-  __shared__ float s_out[kScratchRows * 128];
-  float* sb = s_out + threadIdx.x;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nround; t += stride) {
     StageIn in;
     if (t < n) stage_load<MLP>(a, t, in);
-    const unsigned want = t < n ? stage_one_f32<G, NP, MLP>(a, t, in, c, h32, h64, sb) : 0u;
+    const unsigned want = t < n ? stage_one_f32<G, NP, MLP>(a, t, in, c, h32, h64) : 0u;
     list_append(a.list, a.count, t, want);
   }
   stage_counters(a, c);
@@ -582,7 +578,7 @@ __device__ __forceinline__ unsigned stage_one_f64(const StageArgs& a, int64_t t,
   lagr<NP, double>(xi[0], a.k.sn, a.k.sw, l1);
   lagr<NP, double>(xi[1], a.k.sn, a.k.sw, l2);
   lagr<NP, double>(xi[2], a.k.sn, a.k.sw, l3);
-  interp4<NP, double>(Ue, l1, l2, l3, Uv);
+  interp4<NP>(Ue, l1, l2, l3, Uv);
   particle_accel<G, NP, double>(a.m, a.k, Ue, e, xi, Uv, v, d, tau, st, acc);
   const double As = a.k.A[s], Bs = a.k.B[s], dt = a.dt;
   double xe[3];
