@@ -345,7 +345,7 @@ struct MonoBasis {
 template <int G>
 __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tmask, int nelem,
                        const MonoBasis V, float* __restrict__ hi, float* __restrict__ lo,
-                       float* __restrict__ curv) {
+                       double* __restrict__ m64, float* __restrict__ curv) {
   constexpr int G3 = G * G * G, AP = Mono<G>::AP, CS = Mono<G>::CS;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * nelem) return;
@@ -364,6 +364,23 @@ __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tm
     for (int q = 0; q < n; ++q) w *= 1.1;
     sum += w;
   };
+  double T[G3];
+  for (int q = 0; q < G3; ++q) T[q] = X[3 * q];
+  for (int st = 1; st < G3; st *= G)
+    for (int q = 0; q < G3; ++q) {
+      if ((q / st) % G) continue;
+      double w[G];
+      for (int a = 0; a < G; ++a) w[a] = T[q + a * st];
+      for (int kk = 0; kk < G; ++kk) {
+        double v = 0.0;
+        for (int a = 0; a < G; ++a) v += V.v[kk * G + a] * w[a];
+        T[q + kk * st] = v;
+      }
+    }
+  double* w64 = m64 + (size_t)i * G3;
+  for (int c = 0; c < G; ++c)
+    for (int b = 0; b < G; ++b)
+      for (int a = 0; a < G; ++a) w64[G * (c + G * b) + a] = T[a + G * (b + G * c)];
   if ((tmask[e] >> r) & 1) {  // 8 coefficients of the corner interpolant
     for (int q = 0; q < 8; ++q) {
       double v = 0.0;
@@ -379,19 +396,6 @@ __global__ void k_mono(const double* __restrict__ xg, const int* __restrict__ tm
     curv[4 * (size_t)e + r] = (float)(sum * (1.0 + 1e-6));
     return;
   }
-  double T[G3];
-  for (int q = 0; q < G3; ++q) T[q] = X[3 * q];
-  for (int st = 1; st < G3; st *= G)
-    for (int q = 0; q < G3; ++q) {
-      if ((q / st) % G) continue;
-      double w[G];
-      for (int a = 0; a < G; ++a) w[a] = T[q + a * st];
-      for (int kk = 0; kk < G; ++kk) {
-        double v = 0.0;
-        for (int a = 0; a < G; ++a) v += V.v[kk * G + a] * w[a];
-        T[q + kk * st] = v;
-      }
-    }
   for (int q = 0; q < CS; ++q) h[q] = l[q] = 0.f;
   for (int c = 0; c < G; ++c)
     for (int b = 0; b < G; ++b)
@@ -423,10 +427,10 @@ static cudaError_t launch_mono(pt_ctx* c) {
   }
   const int nb = (3 * c->nelem + 127) / 128;
   switch (c->g) {
-    case 2: k_mono<2><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
-    case 3: k_mono<3><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
-    case 4: k_mono<4><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
-    default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_curv); break;
+    case 2: k_mono<2><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_mono64, c->d_curv); break;
+    case 3: k_mono<3><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_mono64, c->d_curv); break;
+    case 4: k_mono<4><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_mono64, c->d_curv); break;
+    default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_mono64, c->d_curv); break;
   }
   const cudaError_t err = cudaGetLastError();
   return err ? err : cudaStreamSynchronize(c->stream);
@@ -663,6 +667,8 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_monolo = dmalloc<float>(cc, nmono, &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
+  c->d_mono64 = dmalloc<double>(cc, xg64.size(), &err);
+  if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_curv = dmalloc<float>(cc, 4 * (size_t)E, &err);
   if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
   c->d_ce = dmalloc<double>(cc, ce.size(), &err);
@@ -786,6 +792,7 @@ static DevMesh dev_mesh(const pt_ctx* c) {
   m.xg32 = c->d_xg32;
   m.mono = c->d_mono;
   m.monolo = c->d_monolo;
+  m.mono64 = c->d_mono64;
   m.curv = c->d_curv;
   m.ce = c->d_ce;
   m.tri = c->d_tri;

@@ -23,6 +23,7 @@ struct pt_ctx {
   float* d_xg32 = nullptr;
   float* d_mono = nullptr;
   float* d_monolo = nullptr;
+  double* d_mono64 = nullptr;
   float* d_curv = nullptr;
   double* d_ce = nullptr;
   float* d_tri = nullptr;

@@ -164,62 +164,6 @@ __device__ __forceinline__ void matvec3(const T* M, const T* v, T* o) {
 // (FP32 evaluation: pt_map.cuh)
 // ---------------------------------------------------------------------------
 
-// FP64, nodes point-major [G^3][3]; with WJ also the Jacobian
-template <int G, bool WJ>
-__device__ __forceinline__ void map64(const double* __restrict__ X, const double* xi,
-                                      const DevConsts& k, double* chi, double* J) {
-  double l0[G], d0[G], l1[G], d1[G], l2[G], d2[G];
-  if (WJ) {
-    lagr_d<G, double>(xi[0], k.gn, k.gw, l0, d0);
-    lagr_d<G, double>(xi[1], k.gn, k.gw, l1, d1);
-    lagr_d<G, double>(xi[2], k.gn, k.gw, l2, d2);
-  } else {
-    lagr<G, double>(xi[0], k.gn, k.gw, l0);
-    lagr<G, double>(xi[1], k.gn, k.gw, l1);
-    lagr<G, double>(xi[2], k.gn, k.gw, l2);
-  }
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    chi[r] = 0.0;
-    if (WJ) J[3 * r] = J[3 * r + 1] = J[3 * r + 2] = 0.0;
-  }
-#pragma unroll 1
-  for (int c = 0; c < G; ++c) {
-    double T0[3] = {0, 0, 0}, T1[3] = {0, 0, 0}, T2[3] = {0, 0, 0};
-#pragma unroll 1
-    for (int b = 0; b < G; ++b) {
-      double s[3] = {0, 0, 0}, s1[3] = {0, 0, 0};
-#pragma unroll
-      for (int a = 0; a < G; ++a) {
-        const double* P = X + 3 * (a + G * (b + G * c));
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          double xv = __ldg(P + r);
-          s[r] = fma(xv, l0[a], s[r]);
-          if (WJ) s1[r] = fma(xv, d0[a], s1[r]);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        T0[r] = fma(s[r], l1[b], T0[r]);
-        if (WJ) {
-          T1[r] = fma(s1[r], l1[b], T1[r]);
-          T2[r] = fma(s[r], d1[b], T2[r]);
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      chi[r] = fma(T0[r], l2[c], chi[r]);
-      if (WJ) {
-        J[3 * r] = fma(T1[r], l2[c], J[3 * r]);
-        J[3 * r + 1] = fma(T2[r], l2[c], J[3 * r + 1]);
-        J[3 * r + 2] = fma(T0[r], d2[c], J[3 * r + 2]);
-      }
-    }
-  }
-}
-
 // trilinear start xi0 = Jc^{-1} (x_loc - xc), from the per-element table
 __device__ __forceinline__ void trilinear_guess(const DevMesh& m, int e, const float* xf,
                                                 float* xi) {
@@ -230,14 +174,70 @@ __device__ __forceinline__ void trilinear_guess(const DevMesh& m, int e, const f
     xi[q] = __ldg(t + 3 + 3 * q) * r[0] + __ldg(t + 4 + 3 * q) * r[1] + __ldg(t + 5 + 3 * q) * r[2];
 }
 
+// FP64: chi and, with WJ, the Jacobian J[r][q] from the FP64 monomial
+// coefficients M [3][G^3] (row (b, c) at G (c + G b), powers of xi1 in order), by
+// Horner's rule in xi3, xi2 and xi1
+template <int G, bool WJ>
+__device__ __forceinline__ void map64(const double* __restrict__ M, const double* xi, double* chi,
+                                      double* J) {
+  constexpr int G3 = G * G * G;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const double* Mr = M + r * G3;
+    double W[G], Wy[G], Wz[G];
+#pragma unroll
+    for (int b = G - 1; b >= 0; --b) {
+#pragma unroll
+      for (int a = 0; a < G; ++a) {
+        double V = __ldg(Mr + G * (G - 1 + G * b) + a), D = 0.0;
+#pragma unroll
+        for (int c = G - 2; c >= 0; --c) {
+          if (WJ) D = c == G - 2 ? V : fma(D, xi[2], V);
+          V = fma(V, xi[2], __ldg(Mr + G * (c + G * b) + a));
+        }
+        if (b == G - 1) {
+          W[a] = V;
+          if (WJ) Wz[a] = D;
+        } else {
+          if (WJ) {
+            Wy[a] = b == G - 2 ? W[a] : fma(Wy[a], xi[1], W[a]);
+            Wz[a] = fma(Wz[a], xi[1], D);
+          }
+          W[a] = fma(W[a], xi[1], V);
+        }
+      }
+    }
+    double v = W[G - 1], dx = 0.0, dy = 0.0, dz = 0.0;
+    if (WJ) {
+      dy = Wy[G - 1];
+      dz = Wz[G - 1];
+    }
+#pragma unroll
+    for (int a = G - 2; a >= 0; --a) {
+      if (WJ) {
+        dx = a == G - 2 ? v : fma(dx, xi[0], v);
+        dy = fma(dy, xi[0], Wy[a]);
+        dz = fma(dz, xi[0], Wz[a]);
+      }
+      v = fma(v, xi[0], W[a]);
+    }
+    chi[r] = v;
+    if (WJ) {
+      J[3 * r] = dx;
+      J[3 * r + 1] = dy;
+      J[3 * r + 2] = dz;
+    }
+  }
+}
+
 // Full FP64 Newton: chi(xi) - x = 0, |dxi|_inf < tol (Sec. 3.2.1).
 template <int G>
-__device__ __forceinline__ bool newton64(const double* X64, const double* xl, double* xi,
+__device__ __forceinline__ bool newton64(const double* M, const double* xl, double* xi,
                                          const DevConsts& k, int maxit, int& it64) {
   #pragma unroll 1
   for (int it = 0; it < maxit; ++it) {
     double chi[3], J[9], Ji[9], r[3], d[3];
-    map64<G, true>(X64, xi, k, chi, J);
+    map64<G, true>(M, xi, chi, J);
     if (!inv3(J, Ji)) return false;
 #pragma unroll
     for (int q = 0; q < 3; ++q) r[q] = chi[q] - xl[q];
@@ -253,9 +253,73 @@ __device__ __forceinline__ bool newton64(const double* X64, const double* xl, do
 }
 
 template <int G>
-__device__ __noinline__ bool newton64_cold(const double* X64, const double* xl, double* xi,
-                                           const DevConsts& k, int& it64) {
-  return newton64<G>(X64, xl, xi, k, k.max_newton, it64);
+__device__ __noinline__ bool newton64_cold(const double* M, const double* xl, double* xi,
+                                           const DevConsts& k, int maxit, int& it64) {
+  return newton64<G>(M, xl, xi, k, maxit, it64);
+}
+
+// The inverse map of the FP64 mode.  An FP64 instruction holds an SM's FP64
+// unit for 64 cycles per warp, so only what the result's accuracy needs runs in
+// FP64: the start is improved by FP32 Newton iterations (to ~1e-7); one full
+// FP64 Newton step squares that, and the steps after it (one, as a rule, to
+// confirm |dxi| < tol) evaluate the FP64 residual alone and keep the FP64
+// inverse Jacobian of that step, whose relative error is the step's size.  The
+// fixed point is the FP64 residual's zero, as with full Newton steps, which
+// took 3 to 4 evaluations of the FP64 map and Jacobian from the trilinear start
+// and remain the fallback.
+template <int G>
+__device__ __forceinline__ bool newton_f64(const DevMesh& m, const DevConsts& k, int e,
+                                           const double* xl, const float* guess, double* xi,
+                                           int& it64) {
+  const double* M = m.mono64 + (size_t)e * 3 * G * G * G;
+  {
+    const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
+    const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
+    const float xf[3] = {(float)xl[0], (float)xl[1], (float)xl[2]};
+    float z[3] = {guess[0], guess[1], guess[2]};
+    bool ok = true;
+#pragma unroll 1
+    for (int it = 0; it < 6 && ok; ++it) {
+      float chi[3], J[9], Ji[9], r[3], d[3];
+      map_j32<G>(Mh, z, tm, chi, J);
+      if (!inv3(J, Ji)) {
+        ok = false;
+        break;
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) r[q] = chi[q] - xf[q];
+      matvec3(Ji, r, d);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) z[q] -= d[q];
+      ok = tmax3(z[0], z[1], z[2]) <= 4.f;
+      if (tmax3(d[0], d[1], d[2]) < PT_NEWTON_SWITCH) break;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) xi[q] = ok ? z[q] : guess[q];
+  }
+  const int maxit = k.max_newton;
+  double chi[3], Ji[9], r[3], d[3];
+  {
+    double J[9];
+    map64<G, true>(M, xi, chi, J);
+    if (!inv3(J, Ji)) return false;
+  }
+  int it = 0;
+#pragma unroll 1
+  while (true) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) r[q] = chi[q] - xl[q];
+    matvec3(Ji, r, d);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) xi[q] -= d[q];
+    ++it64;
+    ++it;
+    if (tmax3(d[0], d[1], d[2]) < k.newton_tol) return true;
+    if (!(tmax3(xi[0], xi[1], xi[2]) <= 4.0) || it >= maxit) return false;
+    if (it >= 4) break;
+    map64<G, false>(M, xi, chi, nullptr);
+  }
+  return newton64_cold<G>(M, xl, xi, k, maxit - it, it64);
 }
 
 // Mixed-precision Newton on a double-float local position xd (relative to the
@@ -345,7 +409,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
     xi[q] = have ? df_to_double(zd[q]) : (double)guess[q];
   }
   if (!(tmax3(xi[0], xi[1], xi[2]) <= 4.0)) xi[0] = xi[1] = xi[2] = 0.0;
-  const bool ok = newton64_cold<G>(m.xg64 + (size_t)e * 3 * G * G * G, xl, xi, k, it64);
+  const bool ok = newton64_cold<G>(m.mono64 + (size_t)e * 3 * G * G * G, xl, xi, k, k.max_newton, it64);
 #pragma unroll
   for (int q = 0; q < 3; ++q) zd[q] = df_from_double(xi[q]);
   return ok;
@@ -494,25 +558,61 @@ __device__ __forceinline__ void interp4(const float* __restrict__ Ue, const floa
   }
 }
 
-// FP64: sum-factorised
+// FP64 (bound by the FP64 unit): up to N = 5 the weights l1_i l2_j of a plane are
+// formed once for the four variables, a tenth fewer multiply-adds than the sum-
+// factorised form, which larger N keep (the plane's weights would take half
+// the registers); even rows are read 16 bytes at a time
 template <int NP>
 __device__ __forceinline__ void interp4(const double* __restrict__ Ue, const double* l1,
                                         const double* l2, const double* l3, double* out) {
-  constexpr int N3 = NP * NP * NP;
+  constexpr int N2 = NP * NP, N3 = N2 * NP;
+  constexpr bool kW = NP <= 6;
+  double w[kW ? N2 : 1];
+  if constexpr (kW) {
+#pragma unroll
+    for (int q = 0; q < N2; ++q) w[q] = l1[q % NP] * l2[q / NP];
+  }
 #pragma unroll 1
   for (int v = 0; v < 4; ++v) {
-    const double* Uv = Ue + v * N3;
     double acc = 0.0;
 #pragma unroll 1
     for (int kk = 0; kk < NP; ++kk) {
-      double t2 = 0.0;
+      const double* P = Ue + v * N3 + kk * N2;
+      double t2 = 0.0, t3 = 0.0;
+      if constexpr (kW && NP % 2 == 0) {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        const double* row = Uv + NP * (j + NP * kk);
-        double t1 = 0.0;
+        for (int q = 0; q < N2; q += 2) {
+          const double2 u = __ldg(reinterpret_cast<const double2*>(P + q));
+          t2 = fma(u.x, w[q], t2);
+          t3 = fma(u.y, w[q + 1], t3);
+        }
+        t2 += t3;
+      } else if constexpr (kW) {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) t1 = fma(__ldg(row + i), l1[i], t1);
-        t2 = fma(t1, l2[j], t2);
+        for (int q = 0; q < N2; ++q) {
+          if (q & 1)
+            t3 = fma(__ldg(P + q), w[q], t3);
+          else
+            t2 = fma(__ldg(P + q), w[q], t2);
+        }
+        t2 += t3;
+      } else {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          double t1 = 0.0;
+          if constexpr (NP % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < NP; i += 2) {
+              const double2 u = __ldg(reinterpret_cast<const double2*>(P + NP * j + i));
+              t1 = fma(u.x, l1[i], t1);
+              t1 = fma(u.y, l1[i + 1], t1);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) t1 = fma(__ldg(P + NP * j + i), l1[i], t1);
+          }
+          t2 = fma(t1, l2[j], t2);
+        }
       }
       acc = fma(t2, l3[kk], acc);
     }

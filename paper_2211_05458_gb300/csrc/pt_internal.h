@@ -44,6 +44,7 @@ struct DevMesh {
   const float* xg32;      // [E][3][g^3]   nodes - ce, FP32, coordinate-major
   const float* mono;      // [E][3][CS]    monomial coefficients of nodes - ce (pt_map.cuh),
   const float* monolo;    //               high and low FP32 parts
+  const double* mono64;   // [E][3][g^3]   the same in FP64, rows of g
   const float* curv;      // [E][4]        bounds on |second derivatives| of the three
                           //               coordinates of the map for |xi| <= 1.1 (sum over
                           //               a pair of directions; fourth word unused)

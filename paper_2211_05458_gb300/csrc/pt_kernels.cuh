@@ -46,12 +46,7 @@ __device__ __forceinline__ bool locate_one(const DevMesh& m, const DevConsts& k,
                                            int& it32, int& it64) {
   const double* ce = m.ce + 3 * (size_t)e;
   double xl[3] = {x[0] - __ldg(ce), x[1] - __ldg(ce + 1), x[2] - __ldg(ce + 2)};
-  if (F64) {
-    xi[0] = guess[0];
-    xi[1] = guess[1];
-    xi[2] = guess[2];
-    return newton64<G>(m.xg64 + (size_t)e * 3 * G * G * G, xl, xi, k, k.max_newton, it64);
-  }
+  if constexpr (F64) return newton_f64<G>(m, k, e, xl, guess, xi, it64);
   return newton_mixed<G>(m, k, e, xl, guess, xi, it32, it64);
 }
 
@@ -60,12 +55,7 @@ template <int G, bool F64>
 __device__ __forceinline__ bool locate_local(const DevMesh& m, const DevConsts& k, int e,
                                              const double* xl, const float* guess, double* xi,
                                              int& it32, int& it64) {
-  if (F64) {
-    xi[0] = guess[0];
-    xi[1] = guess[1];
-    xi[2] = guess[2];
-    return newton64<G>(m.xg64 + (size_t)e * 3 * G * G * G, xl, xi, k, k.max_newton, it64);
-  }
+  if constexpr (F64) return newton_f64<G>(m, k, e, xl, guess, xi, it64);
   return newton_mixed<G>(m, k, e, xl, guess, xi, it32, it64);
 }
 
@@ -168,7 +158,7 @@ __device__ __noinline__ void saffman_force(const DevMesh& m, const DevConsts& k,
     map_j32<G>(m.mono + (size_t)e * 3 * Mono<G>::CS, xf, __ldg(m.tmask + e), chi, J);
   } else {
     double chi[3];
-    map64<G, true>(m.xg64 + (size_t)e * 3 * G3, xi, k, chi, J);
+    map64<G, true>(m.mono64 + (size_t)e * 3 * G3, xi, chi, J);
   }
   F[0] = F[1] = F[2] = T(0);
   if (!inv3(J, Ji)) return;
@@ -341,11 +331,7 @@ __device__ __noinline__ int settle64(const DevMesh& m, const DevConsts& k, int& 
       const float xf[3] = {(float)xl[0], (float)xl[1], (float)xl[2]};
       float g[3];
       trilinear_guess(m, e, xf, g);
-      xi[0] = g[0];
-      xi[1] = g[1];
-      xi[2] = g[2];
-      if (!newton64<G>(m.xg64 + (size_t)e * 3 * G * G * G, xl, xi, k, k.max_newton, it64))
-        return 1;
+      if (!newton_f64<G>(m, k, e, xl, g, xi, it64)) return 1;
     }
     have = false;
     if (tmax3(xi[0], xi[1], xi[2]) <= 1.0 + wtol) return 0;
@@ -953,7 +939,7 @@ __device__ __forceinline__ bool particle_source(const DepositArgs& a, int64_t ip
     }
     const double xn[3] = {a.k.sn[id[0]], a.k.sn[id[1]], a.k.sn[id[2]]};
     double chi[3], J[9];
-    map64<G, true>(a.m.xg64 + (size_t)e * G * G * G * 3, xn, a.k, chi, J);
+    map64<G, true>(a.m.mono64 + (size_t)e * G * G * G * 3, xn, chi, J);
     const double det = J[0] * (J[4] * J[8] - J[5] * J[7]) - J[1] * (J[3] * J[8] - J[5] * J[6]) +
                        J[2] * (J[3] * J[7] - J[4] * J[6]);
     const R iv = R(1) / (R)(a.k.sq[id[0]] * a.k.sq[id[1]] * a.k.sq[id[2]] * fabs(det));

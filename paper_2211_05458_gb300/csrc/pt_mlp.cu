@@ -144,14 +144,14 @@ __global__ void k_mlp_pairs(DevMesh m, DevConsts k, int64_t n, uint64_t seed, co
   const int e = (int)(splitmix64(base + 1) % (uint64_t)m.nelem);
   double xi_true[3];
   for (int q = 0; q < 3; ++q) xi_true[q] = 2.0 * u01(splitmix64(base + 2 + q)) - 1.0;
-  const double* X64 = m.xg64 + (size_t)e * 3 * G * G * G;
+  const double* M = m.mono64 + (size_t)e * 3 * G * G * G;
   double xl[3];
-  pt::map64<G, false>(X64, xi_true, k, xl, nullptr);
+  pt::map64<G, false>(M, xi_true, xl, nullptr);
   float xf[3] = {(float)xl[0], (float)xl[1], (float)xl[2]}, g[3];
   pt::trilinear_guess(m, e, xf, g);
   double xi[3] = {g[0], g[1], g[2]};
   int it = 0;
-  bool ok = pt::newton64<G>(X64, xl, xi, k, k.max_newton, it);
+  bool ok = pt::newton64<G>(M, xl, xi, k, k.max_newton, it);
   if (!ok) {
     atomicAdd(nfail, 1u);
     for (int q = 0; q < 3; ++q) xi[q] = xi_true[q];
