@@ -328,12 +328,17 @@ __device__ __forceinline__ bool newton_f64(const DevMesh& m, const DevConsts& k,
 // the step is below newton_tol.  Returns the double-float xi in zd and, unless
 // the (out-of-line) fallback of a full FP64 Newton was taken (jok false), the
 // inverse Jacobian at xi to ~1e-5 in Ji.
-template <int G>
+// GEN: the element's coefficients (high, low parts) may be in shared memory,
+// at Mh and Ml.
+template <int G, bool GEN = false>
 __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, int e,
                                           const df* xd, const float* guess, df* zd, int& it32,
-                                          int& it64, float* Ji, bool& jok) {
-  const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
-  const float* Ml = m.monolo + (size_t)e * 3 * Mono<G>::CS;
+                                          int& it64, float* Ji, bool& jok,
+                                          const float* Mh = nullptr, const float* Ml = nullptr) {
+  if constexpr (!GEN) {
+    Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
+    Ml = m.monolo + (size_t)e * 3 * Mono<G>::CS;
+  }
   const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
   float z[3] = {guess[0], guess[1], guess[2]};
   bool have = false;
@@ -341,7 +346,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
   #pragma unroll 1
   for (int it = 0; it < 8; ++it) {
     float chi[3], J[9], r[3], d[3];
-    map_j32<G>(Mh, z, tm, chi, J);
+    map_j32<G, GEN>(Mh, z, tm, chi, J);
     if (!inv3(J, Ji)) break;
     have = true;
 #pragma unroll
@@ -374,14 +379,14 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
       float r[3], d[3], zm[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) zm[q] = inc ? fmaf(0.5f, dz[q], z[q]) : zd[q].hi;
-      if (!inc) resid_df<G>(Mh, Ml, zm, tm, xd, rp);
+      if (!inc) resid_df<G, GEN>(Mh, Ml, zm, tm, xd, rp);
 #pragma unroll
       for (int q = 0; q < 3; ++q) r[q] = rp[q];
       if (it > 0) {
         float chi[3], J[9], Jd[3];
         const float by[3] = {inc ? dz[0] : zd[0].lo, inc ? dz[1] : zd[1].lo,
                              inc ? dz[2] : zd[2].lo};
-        map_j32<G>(Mh, zm, tm, chi, J);
+        map_j32<G, GEN>(Mh, zm, tm, chi, J);
         matvec3(J, by, Jd);
 #pragma unroll
         for (int q = 0; q < 3; ++q) r[q] += Jd[q];
@@ -449,7 +454,7 @@ __device__ __forceinline__ bool newton_mixed(const DevMesh& m, const DevConsts& 
 // room for fewer loads: 312 against 235 us per stage of 10^6 particles).  The
 // third-direction basis is shifted through registers by the rolled loop, which
 // keeps it out of local memory.
-template <int NP>
+template <int NP, bool GEN = false>
 __device__ __forceinline__ void interp4(const float* __restrict__ Ue, const float* l1,
                                         const float* l2, const float* l3, float* out) {
   constexpr int N2 = NP * NP, N3 = N2 * NP, NH = NP / 2;
@@ -484,7 +489,7 @@ __device__ __forceinline__ void interp4(const float* __restrict__ Ue, const floa
               reinterpret_cast<const ulonglong2*>(Ue + (v + q) * N3 + kk * N2);
 #pragma unroll
           for (int i = 0; i < N2 / 4; ++i) {
-            const ulonglong2 x = __ldg(P + i);
+            const ulonglong2 x = ldx<GEN>(P + i);
             u[q][2 * i] = x.x;
             u[q][2 * i + 1] = x.y;
           }
@@ -542,7 +547,7 @@ __device__ __forceinline__ void interp4(const float* __restrict__ Ue, const floa
           f32x2 t1;
 #pragma unroll
           for (int i = 0; i < NP; ++i) {
-            const f32x2 x = pk2(__ldg(P + j * NP + i), __ldg(P + N3 + j * NP + i));
+            const f32x2 x = pk2(ldx<GEN>(P + j * NP + i), ldx<GEN>(P + N3 + j * NP + i));
             t1 = i ? fma2(x, dup2(l1[i]), t1) : mul2(x, dup2(l1[0]));
           }
           t = j ? fma2(t1, w2[j], t) : mul2(t1, w2[0]);

@@ -352,10 +352,11 @@ __device__ __noinline__ int settle64(const DevMesh& m, const DevConsts& k, int& 
 }
 
 // FP32 mode: xd local double-float position in element e, zd its xi (valid
-// on entry if have).
+// on entry if have); Ji, jok as newton_df's, of the last inverse map.
 template <int G>
 __device__ __noinline__ int settle_f32(const DevMesh& m, const DevConsts& k, int& e, df* xd,
-                                       df* zd, bool have, int& it32, int& it64, int& cross) {
+                                       df* zd, bool have, int& it32, int& it64, int& cross,
+                                       float* Ji, bool& jok) {
   const double wtol = settle_tol(k);
 #pragma unroll 1
   for (int w = 0; w <= 4; ++w) {
@@ -363,7 +364,7 @@ __device__ __noinline__ int settle_f32(const DevMesh& m, const DevConsts& k, int
       const float xf[3] = {xd[0].hi, xd[1].hi, xd[2].hi};
       float g[3];
       trilinear_guess(m, e, xf, g);
-      if (!newton_df<G>(m, k, e, xd, g, zd, it32, it64)) return 1;
+      if (!newton_df<G>(m, k, e, xd, g, zd, it32, it64, Ji, jok)) return 1;
     }
     have = false;
     if (tmax3(zd[0].hi, zd[1].hi, zd[2].hi) < 1.f - 1e-5f) return 0;  // decided in FP32
@@ -446,9 +447,8 @@ __device__ __forceinline__ void push_particle(const DevMesh& m, const DevConsts&
       start_guess_local<G, MLP>(m, k, sm, mlpp, eg, xf, live, guess);
       if (!live) continue;
       double xi[3];
-      int i32 = 0, i64 = 0;
-      bool ok = locate_local<G, F64>(m, k, e, xl, guess, xi, i32, i64);
-      c.it32 += i32;
+      int i64 = 0;
+      const bool ok = newton_f64<G>(m, k, e, xl, guess, xi, i64);
       c.it64 += i64;
       if (!ok) {
         st |= PT_ST_NEWTON_FAIL;
@@ -617,7 +617,7 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
         }
         if (md > 1.0 + settle_tol(k) && pending) {
           int cr = 0, j32 = 0, j64 = 0;
-          const int rc = settle_f32<G>(m, k, e, xd, zd, true, j32, j64, cr);
+          const int rc = settle_f32<G>(m, k, e, xd, zd, true, j32, j64, cr, Ji, jok);
           c.it32 += j32;
           c.it64 += j64;
           c.tc.cross += cr;
@@ -626,7 +626,6 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
             live = false;
             continue;
           }
-          jok = false;  // Ji belongs to the element left
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
             xi[q] = zd[q].hi + zd[q].lo;
@@ -705,8 +704,10 @@ __device__ __forceinline__ void push_particle_f32(const DevMesh& m, const DevCon
   }
   if (live && pending) {
     df zd[3];
+    float Ji[9];
+    bool jok;
     int cr = 0, j32 = 0, j64 = 0;
-    const int rc = settle_f32<G>(m, k, e, xd, zd, false, j32, j64, cr);
+    const int rc = settle_f32<G>(m, k, e, xd, zd, false, j32, j64, cr, Ji, jok);
     c.it32 += j32;
     c.it64 += j64;
     c.tc.cross += cr;
@@ -1366,6 +1367,14 @@ struct Family {
       case PT_SOP_STAGE:
         if constexpr (F64) {
           k_stage_f64<G, NP><<<grid, block, 0, s>>>(a);
+        } else if (ElemSlot<G, NP>::ok && a.n >= 24 * (int64_t)a.m.nelem) {
+          if constexpr (ElemSlot<G, NP>::ok) {
+            constexpr int dyn = ElemSlot<G, NP>::bytes;  // at most 44 KB: no attribute needed
+            if (kMlp && a.k.guess == PT_GUESS_MLP)
+              k_stage_sm_f32<G, NP, kMlp><<<grid, block, dyn, s>>>(a);
+            else
+              k_stage_sm_f32<G, NP, false><<<grid, block, dyn, s>>>(a);
+          }
         } else if (kMlp && a.k.guess == PT_GUESS_MLP) {
           k_stage_f32<G, NP, kMlp><<<grid, block, 0, s>>>(a);
         } else {

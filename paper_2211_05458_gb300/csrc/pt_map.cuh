@@ -34,24 +34,35 @@ struct Mono {
   static constexpr int CS = (G * G * AP + 3) & ~3;
 };
 
+// Read-only load: non-coherent from global memory, or (GEN) generic, for data
+// that may sit in shared memory.
+template <bool GEN, typename V>
+__device__ __forceinline__ V ldx(const V* p) {
+  if constexpr (GEN)
+    return *p;
+  else
+    return __ldg(p);
+}
+
 // one row as packed pairs
-template <int G>
+template <int G, bool GEN>
 __device__ __forceinline__ void mono_row(const float* __restrict__ p, f32x2* q) {
   if constexpr (Mono<G>::AP == 4) {
-    const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(p));
+    const ulonglong2 w = ldx<GEN>(reinterpret_cast<const ulonglong2*>(p));
     q[0] = w.x;
     q[1] = w.y;
   } else {
 #pragma unroll
-    for (int i = 0; i < Mono<G>::NQ; ++i) q[i] = __ldg(reinterpret_cast<const f32x2*>(p) + i);
+    for (int i = 0; i < Mono<G>::NQ; ++i) q[i] = ldx<GEN>(reinterpret_cast<const f32x2*>(p) + i);
   }
 }
 
 // chi_r and its three derivatives of a trilinear coordinate
+template <bool GEN>
 __device__ __forceinline__ void mono_tri32(const float* __restrict__ M, const float* xi, float& chi,
                                            float* J) {
-  const ulonglong2 q0 = __ldg(reinterpret_cast<const ulonglong2*>(M));
-  const ulonglong2 q1 = __ldg(reinterpret_cast<const ulonglong2*>(M) + 1);
+  const ulonglong2 q0 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(M));
+  const ulonglong2 q1 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(M) + 1);
   const f32x2 z = dup2(xi[2]), y = dup2(xi[1]);
   const f32x2 s0 = fma2(z, q1.x, q0.x), s1 = fma2(z, q1.y, q0.y);  // b = 0, 1
   float u0, u1, v0, v1, w0, w1;
@@ -66,7 +77,7 @@ __device__ __forceinline__ void mono_tri32(const float* __restrict__ M, const fl
 
 // the same for a curved coordinate: Horner in xi3, then xi2 (packed over the
 // powers of xi1), then xi1, each with its derivative
-template <int G>
+template <int G, bool GEN>
 __device__ __forceinline__ void mono_curved32(const float* __restrict__ M, const float* xi,
                                               float& chi, float* J) {
   constexpr int AP = Mono<G>::AP, NQ = Mono<G>::NQ;
@@ -76,7 +87,7 @@ __device__ __forceinline__ void mono_curved32(const float* __restrict__ M, const
   for (int b = G - 1; b >= 0; --b) {
     f32x2 row[G][NQ];
 #pragma unroll
-    for (int c = 0; c < G; ++c) mono_row<G>(M + AP * (c + G * b), row[c]);
+    for (int c = 0; c < G; ++c) mono_row<G, GEN>(M + AP * (c + G * b), row[c]);
 #pragma unroll
     for (int p = 0; p < NQ; ++p) {
       f32x2 V = fma2(row[G - 1][p], z, row[G - 2][p]), D = row[G - 1][p];
@@ -118,16 +129,16 @@ __device__ __forceinline__ void mono_curved32(const float* __restrict__ M, const
 
 // chi and Jacobian J[r][q] = d chi_r / d xi_q in FP32; M: the element's
 // coefficients (high parts), tm: its trilinear coordinates
-template <int G>
+template <int G, bool GEN = false>
 __device__ __forceinline__ void map_j32(const float* __restrict__ M, const float* xi, int tm,
                                         float* chi, float* J) {
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const float* Mr = M + r * Mono<G>::CS;
     if (G == 2 || ((tm >> r) & 1))
-      mono_tri32(Mr, xi, chi[r], J + 3 * r);
+      mono_tri32<GEN>(Mr, xi, chi[r], J + 3 * r);
     else if constexpr (G > 2)
-      mono_curved32<G>(Mr, xi, chi[r], J + 3 * r);
+      mono_curved32<G, GEN>(Mr, xi, chi[r], J + 3 * r);
   }
 }
 
@@ -155,12 +166,13 @@ __device__ __forceinline__ void comp_step(float& s, float& e, float z, float h, 
 }
 
 // chi_r(xi) of one coordinate as s + e, xi three FP32 numbers
+template <bool GEN>
 __device__ __forceinline__ void comp_tri(const float* __restrict__ Mh, const float* __restrict__ Ml,
                                          const float* xi, float& s, float& e) {
-  const ulonglong2 h0 = __ldg(reinterpret_cast<const ulonglong2*>(Mh));
-  const ulonglong2 h1 = __ldg(reinterpret_cast<const ulonglong2*>(Mh) + 1);
-  const ulonglong2 l0 = __ldg(reinterpret_cast<const ulonglong2*>(Ml));
-  const ulonglong2 l1 = __ldg(reinterpret_cast<const ulonglong2*>(Ml) + 1);
+  const ulonglong2 h0 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(Mh));
+  const ulonglong2 h1 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(Mh) + 1);
+  const ulonglong2 l0 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(Ml));
+  const ulonglong2 l1 = ldx<GEN>(reinterpret_cast<const ulonglong2*>(Ml) + 1);
   const f32x2 z = dup2(xi[2]), zn = dup2(-xi[2]), y = dup2(xi[1]), yn = dup2(-xi[1]);
   f32x2 s0 = h1.x, e0 = l1.x, s1 = h1.y, e1 = l1.y;
   comp_step(s0, e0, z, zn, h0.x, l0.x);
@@ -174,7 +186,7 @@ __device__ __forceinline__ void comp_tri(const float* __restrict__ Mh, const flo
   e = b1;
 }
 
-template <int G>
+template <int G, bool GEN>
 __device__ __forceinline__ void comp_curved(const float* __restrict__ Mh,
                                             const float* __restrict__ Ml, const float* xi,
                                             float& so, float& eo) {
@@ -184,13 +196,13 @@ __device__ __forceinline__ void comp_curved(const float* __restrict__ Mh,
 #pragma unroll
   for (int b = G - 1; b >= 0; --b) {
     f32x2 s[NQ], e[NQ];
-    mono_row<G>(Mh + AP * (G - 1 + G * b), s);
-    mono_row<G>(Ml + AP * (G - 1 + G * b), e);
+    mono_row<G, GEN>(Mh + AP * (G - 1 + G * b), s);
+    mono_row<G, GEN>(Ml + AP * (G - 1 + G * b), e);
 #pragma unroll
     for (int c = G - 2; c >= 0; --c) {
       f32x2 h[NQ], l[NQ];
-      mono_row<G>(Mh + AP * (c + G * b), h);
-      mono_row<G>(Ml + AP * (c + G * b), l);
+      mono_row<G, GEN>(Mh + AP * (c + G * b), h);
+      mono_row<G, GEN>(Ml + AP * (c + G * b), l);
 #pragma unroll
       for (int p = 0; p < NQ; ++p) comp_step(s[p], e[p], z, zn, h[p], l[p]);
     }
@@ -219,7 +231,7 @@ __device__ __forceinline__ void comp_curved(const float* __restrict__ Mh,
 // Residual chi(xi) - x at an FP32 point xi, x a double-float; the difference
 // of the high parts is exact where they agree to a factor of two, which is
 // where the residual's accuracy counts.
-template <int G>
+template <int G, bool GEN = false>
 __device__ __forceinline__ void resid_df(const float* __restrict__ Mh, const float* __restrict__ Ml,
                                          const float* xi, int tm, const df* x, float* r) {
 #pragma unroll
@@ -228,9 +240,9 @@ __device__ __forceinline__ void resid_df(const float* __restrict__ Mh, const flo
     const float* l = Ml + q * Mono<G>::CS;
     float s = 0.f, e = 0.f;
     if (G == 2 || ((tm >> q) & 1))
-      comp_tri(h, l, xi, s, e);
+      comp_tri<GEN>(h, l, xi, s, e);
     else if constexpr (G > 2)
-      comp_curved<G>(h, l, xi, s, e);
+      comp_curved<G, GEN>(h, l, xi, s, e);
     r[q] = __fadd_rn(__fsub_rn(s, x[q].hi), __fsub_rn(e, x[q].lo));
   }
 }

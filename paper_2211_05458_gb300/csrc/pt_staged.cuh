@@ -135,17 +135,30 @@ __device__ __forceinline__ void stage_load(const StageArgs& a, int64_t t, StageI
 
 // Returns 0 (stage end committed), 1 (listed for exact tracking) or 2 (listed
 // for the walk only).
-template <int G, int NP, bool MLP>
+// SM: Es points at the element's data (ElemSlot) in shared memory, or is null
+// for an element that has no slot.
+template <int G, int NP, bool MLP, bool SM = false>
 __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
                                                   const StageIn& in, PushCounters& c, Hist8& h32,
-                                                  Hist8& h64) {
+                                                  Hist8& h64, const float* Es = nullptr) {
   constexpr int N3 = NP * NP * NP;
   const int64_t n = a.n;
   const int s = a.stage;
   unsigned st = in.st;
   if (st & PT_ST_FROZEN) return 0u;
   const int e = in.e;
-  if constexpr (!MLP) prefetch_element<G, NP>(a, e);
+  if constexpr (!MLP && !SM) prefetch_element<G, NP>(a, e);
+  const float* Mh = a.m.mono + (size_t)e * 3 * Mono<G>::CS;
+  const float* Ml = a.m.monolo + (size_t)e * 3 * Mono<G>::CS;
+  const float* Ue = reinterpret_cast<const float*>(a.U) + (size_t)e * 5 * N3;
+  const float* Ui = Ue;
+  if constexpr (SM) {
+    if (Es) {
+      Mh = Es;
+      Ml = Es + 3 * Mono<G>::CS;
+      Ui = Es + 6 * Mono<G>::CS;
+    }
+  }
   float* vg = reinterpret_cast<float*>(a.v);
   float* kxg = reinterpret_cast<float*>(a.kx);
   float* kvg = reinterpret_cast<float*>(a.kv);
@@ -172,7 +185,7 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
   int i32 = 0, i64 = 0;
   float Ji[9];
   bool jok;
-  const bool ok = newton_df<G>(a.m, a.k, e, xd, guess, zd, i32, i64, Ji, jok);
+  const bool ok = newton_df<G, SM>(a.m, a.k, e, xd, guess, zd, i32, i64, Ji, jok, Mh, Ml);
   c.it32 += i32;
   c.it64 += i64;
   h32.add(i32);
@@ -193,12 +206,11 @@ __device__ __forceinline__ unsigned stage_one_f32(const StageArgs& a, int64_t t,
     if (md > 1.0 - a.k.band_ref) st |= near_bits(a.m, e, z, a.k.band_ref);
   }
   // interpolation of rho, rho u at xi, drag + gravity
-  const float* Ue = reinterpret_cast<const float*>(a.U) + (size_t)e * 5 * N3;
   float l1[NP], l2[NP], l3[NP], Uv[4], acc[3];
   lagr<NP, float>(xi[0], a.k.sn32, a.k.sw32, l1);
   lagr<NP, float>(xi[1], a.k.sn32, a.k.sw32, l2);
   lagr<NP, float>(xi[2], a.k.sn32, a.k.sw32, l3);
-  interp4<NP>(Ue, l1, l2, l3, Uv);
+  interp4<NP, SM>(Ui, l1, l2, l3, Uv);
   particle_accel_f32<G, NP>(a.m, a.k, Ue, e, zd, Uv, v, d, tau, st, acc);
   const float As = a.k.A32[s], Bs = a.k.B32[s], dt = a.dt32;
   df xe[3];
@@ -266,6 +278,118 @@ __global__ void __launch_bounds__(128, PT_STAGE_MINB) k_stage_f32(const __grid_c
   h64.flush(a.stats, PT_C_H64, 8);
 }
 
+// Element slots: per warp two copies of an element's data in shared memory --
+// map coefficients, high then low parts (3 CS floats each), and rho, rho u
+// (4 NP^3) -- for the two owners most of the warp's 32 sorted particles share.
+template <int G, int NP>
+struct ElemSlot {
+  static constexpr int F = 6 * Mono<G>::CS + 4 * NP * NP * NP;  // floats, a multiple of 4
+  static constexpr int bytes = 4 * 2 * F * 4;                    // block of 4 warps
+  // bulk copies need 16-byte aligned blocks of the state (even NP); four blocks
+  // per SM must leave L1 some room
+  static constexpr bool ok = NP % 2 == 0 && bytes <= 45056;
+};
+
+// bounded wait without reading a clock: a try may suspend the thread
+__device__ __forceinline__ bool slot_wait(uint32_t mbar, uint32_t parity) {
+#pragma unroll 1
+  for (int k = 0; k < (1 << 20); ++k) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// As k_stage_f32, with the element data of each warp's first two owners copied
+// to shared memory by bulk copies as soon as the owners are known.  The stage is
+// bound by load latency: through L1 every row of the coefficients and of the
+// state that the warp touches first is a round trip to L2, some 30 in a row per
+// particle; the copies make that one.  A lane whose owner has no slot (a third
+// owner, a particle that has crossed since the binning) reads global memory
+// through the same generic loads.  us per stage against k_stage_f32: 203 / 240
+// (10^6 particles, 30 per element, NGeo 2, N 5), 964 / 1078 (4.2e6, 38 per
+// element, NGeo 3, N 5, learned start), 73 / 86 (5e5, 36, NGeo 2, N 3).  With
+// fewer particles per element a warp meets more owners than slots (NGeo 2, N 5:
+// 425 / 520 at 37.5 per element, 306 / 295 at 18.8, 210 / 183 at 9.4; NGeo 3,
+// N 3: 381 / 405, 259 / 231, 168 / 142): used from 24 per element on.
+template <int G, int NP, bool MLP>
+__global__ void __launch_bounds__(128, PT_STAGE_MINB) k_stage_sm_f32(const __grid_constant__ StageArgs a) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_next = *a.count2_next = 0u;
+  constexpr int CS = Mono<G>::CS, N3 = NP * NP * NP, F = ElemSlot<G, NP>::F;
+  extern __shared__ __align__(128) float s_el[];
+  __shared__ unsigned long long s_bar[4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* slots = s_el + w * 2 * F;
+  const uint32_t mb = smem_u32(s_bar + w);
+  if (lane == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mb) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncwarp();
+  uint32_t phase = 0u;
+  bool dead = false;  // a copy did not arrive in time: no more slots for this warp
+  PushCounters c = {0, 0, 0, {0, 0, 0}};
+  Hist8 h32, h64;
+  const int64_t n = a.n;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t nround = (n + stride - 1) / stride * stride;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nround; t += stride) {
+    StageIn in;
+    if (t < n) stage_load<MLP>(a, t, in);
+    const int e0 = (t < n && !(in.st & PT_ST_FROZEN)) ? in.e : -1;
+    // the first owner, and the first that differs from it
+    const unsigned m0 = __ballot_sync(0xffffffffu, e0 >= 0);
+    const int ea = __shfl_sync(0xffffffffu, e0, m0 ? __ffs(m0) - 1 : 0);
+    const unsigned m1 = __ballot_sync(0xffffffffu, e0 >= 0 && e0 != ea);
+    const int eb = __shfl_sync(0xffffffffu, e0, m1 ? __ffs(m1) - 1 : 0);
+    const int ns = dead || !m0 ? 0 : (m1 ? 2 : 1);
+    const float* Es = nullptr;
+    if (ns) {
+      fence_async_smem();  // the lanes' reads of the slots come before the copies
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mb),
+                     "r"(ns * F * 4)
+                     : "memory");
+      __syncwarp();
+      if (lane < 3 * ns) {
+        const int q = lane >= 3, part = lane - 3 * q;
+        const int e = q ? eb : ea;
+        const float* src = part == 0   ? a.m.mono + (size_t)e * 3 * CS
+                           : part == 1 ? a.m.monolo + (size_t)e * 3 * CS
+                                       : reinterpret_cast<const float*>(a.U) + (size_t)e * 5 * N3;
+        const float* dst = slots + q * F + 3 * CS * part;
+        const uint32_t bytes = part < 2 ? 12 * CS : 16 * N3;
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+            "[%3];\n" ::"r"(smem_u32(dst)),
+            "l"(src), "r"(bytes), "r"(mb)
+            : "memory");
+      }
+      const bool done = slot_wait(mb, phase);
+      if (__any_sync(0xffffffffu, !done)) {
+        if (!slot_wait(mb, phase)) dead = true;
+        dead = __any_sync(0xffffffffu, dead);
+        if (dead && lane == 0) atomicAdd(a.stats + PT_C_TIMEOUT, 1ull);
+      }
+      phase ^= 1u;
+      if (!dead && e0 >= 0) Es = e0 == ea ? slots : (e0 == eb ? slots + F : nullptr);
+    }
+    const unsigned want =
+        t < n ? stage_one_f32<G, NP, MLP, true>(a, t, in, c, h32, h64, Es) : 0u;
+    list_append(a.list, a.count, t, want);
+  }
+  stage_counters(a, c);
+  h32.flush(a.stats, PT_C_H32, 8);
+  h64.flush(a.stats, PT_C_H64, 8);
+}
+
 // The listed stage segments, first pass: tracking in reference space (track_f32)
 // or the walk.  Segments that it does not decide (walls, open and mortar faces,
 // ends and edges within the bands) go to a second list for k_exact_f32, so that
@@ -305,7 +429,9 @@ __global__ void __launch_bounds__(64, 4) k_track_f32(const __grid_constant__ Sta
         if (bits) a.st[t] |= bits;
       } else {
         df zd[3];
-        rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr);
+        float Ji[9];
+        bool jok;
+        rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr, Ji, jok);
       }
       c.it32 += j32;
       c.it64 += j64;
@@ -374,8 +500,10 @@ __global__ void __launch_bounds__(32) k_exact_f32(const __grid_constant__ StageA
     for (int r = 0; r < 3; ++r) xd[r] = df_from_double(xs[r] - __ldg(cn + r));
     if (!(st & PT_ST_FROZEN)) {
       df zd[3];
+      float Ji[9];
+      bool jok;
       int cr = 0, j32 = 0, j64 = 0;
-      const int rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr);
+      const int rc = settle_f32<G>(a.m, a.k, e, xd, zd, false, j32, j64, cr, Ji, jok);
       c.it32 += j32;
       c.it64 += j64;
       c.tc.cross += cr;
@@ -558,9 +686,8 @@ __device__ __forceinline__ unsigned stage_one_f64(const StageArgs& a, int64_t t,
   float guess[3];
   trilinear_guess(a.m, e, xf, guess);
   double xi[3];
-  int i32 = 0, i64 = 0;
-  const bool ok = locate_local<G, true>(a.m, a.k, e, xl, guess, xi, i32, i64);
-  c.it32 += i32;
+  int i64 = 0;
+  const bool ok = newton_f64<G>(a.m, a.k, e, xl, guess, xi, i64);
   c.it64 += i64;
   h64.add(i64);
   if (!ok) {
