@@ -133,14 +133,42 @@ __device__ void block_bitonic(int* a, unsigned m) {
 }
 
 constexpr int kSortSmem = 4096;  // segments up to this size are sorted in shared memory
+constexpr int kSortWarp = 128;   // segments up to this size are sorted by one warp
 
+// Segments of at most kSortWarp particles, one warp each: a particle's place is
+// the number of smaller indices in its segment (they are distinct), counted
+// over the segment in shared memory without any barrier of the block.  The
+// usual segment holds a few dozen particles, for which the bitonic network's
+// ~20 block barriers cost more than the m^2 / 32 comparisons.
+__global__ void __launch_bounds__(256) k_rank_segments(const int* __restrict__ perm,
+                                                       const int* __restrict__ offs, int nbins,
+                                                       int* __restrict__ out) {
+  __shared__ int sh[8][kSortWarp];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* v = sh[w];
+  for (int e = blockIdx.x * 8 + w; e < nbins; e += gridDim.x * 8) {
+    const int beg = offs[e], m = offs[e + 1] - beg;
+    if (m <= 0 || m > kSortWarp) continue;
+    for (int i = lane; i < m; i += 32) v[i] = perm[beg + i];
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {
+      const int x = v[i];
+      int r = 0;
+      for (int j = 0; j < m; ++j) r += v[j] < x ? 1 : 0;
+      out[beg + r] = x;
+    }
+    __syncwarp();
+  }
+}
+
+// Larger segments, one block each: a bitonic network
 __global__ void __launch_bounds__(256) k_sort_segments(const int* __restrict__ perm,
                                                        const int* __restrict__ offs, int nbins,
                                                        int* out) {
   __shared__ int sh[kSortSmem];
   for (int e = blockIdx.x; e < nbins; e += gridDim.x) {
     const int beg = offs[e], m = offs[e + 1] - beg;
-    if (m <= 0) continue;
+    if (m <= kSortWarp) continue;
     if (m <= kSortSmem) {
       for (int i = threadIdx.x; i < m; i += blockDim.x) sh[i] = perm[beg + i];
       __syncthreads();
@@ -160,6 +188,8 @@ __global__ void __launch_bounds__(256) k_sort_segments(const int* __restrict__ p
 int sort_segments(const int* perm, const int* offs, int nelem, int* out, int nsm,
                   cudaStream_t s) {
   const int nbins = nelem + 1;
+  const int gw = (nbins + 7) / 8 < nsm * 8 ? (nbins + 7) / 8 : nsm * 8;
+  k_rank_segments<<<gw, 256, 0, s>>>(perm, offs, nbins, out);
   const int g = nbins < nsm * 8 ? nbins : nsm * 8;
   k_sort_segments<<<g > 0 ? g : 1, 256, 0, s>>>(perm, offs, nbins, out);
   return (int)cudaGetLastError();
