@@ -81,9 +81,9 @@ typedef enum { PT_TRACK_PHYSICAL = 0, PT_TRACK_REFERENCE = 1 } pt_track;
  * stage over the particle state in element-sorted order (held in library-
  * owned device buffers of about 116 bytes per particle in PT_FP32 mode, 144 in
  * PT_FP64 mode), the stage segments that may cross a face collected in a
- * compacted list and intersected by a second kernel on full warps.  AUTO:
- * STAGED from 2^18 particles on, RESIDENT below (launch latency dominates
- * small pushes).  Both run the same arithmetic in the same order per
+ * compacted list and tracked by kernels of their own.  AUTO: STAGED from
+ * 2^19 particles on (2^18 with the learned start), RESIDENT below (the list
+ * kernels' latency dominates small pushes).  Both run the same arithmetic in the same order per
  * particle. */
 typedef enum { PT_SCHEDULE_AUTO = 0, PT_SCHEDULE_RESIDENT = 1, PT_SCHEDULE_STAGED = 2 } pt_schedule;
 typedef enum {
@@ -145,7 +145,7 @@ typedef struct {
   int32_t max_newton;   /* Newton iteration cap (default 50)                       */
   int32_t max_cross;    /* face-crossing cap per RK stage (default 64)             */
   int32_t rebin_every;  /* steps between particle re-binning; 0 = library choice   */
-  int32_t block;        /* threads per block of the push kernel (32..128); 0 = 128 */
+  int32_t block;        /* threads per block of the push kernel (32..128); 0 = library choice */
   int32_t lift;         /* 1: add the Saffman lift with Mei's correction (Sec. 2.2),
                            F_S = 6.46/4 C_S d^2 sqrt(rho mu/|w|) (u - v) x w, w = curl u;
                            also deposited by pt_deposit (default 0)                */
@@ -301,8 +301,8 @@ pt_status pt_push_host(pt_ctx* ctx, const pt_particles* p_host, int32_t nsteps, 
  * of the element volume (the paper's projection operator).  Summation:
  * PT_DEPOSIT_ATOMIC adds with FP32 atomics (order-dependent rounding);
  * PT_DEPOSIT_SEGMENTED sums each element's particles in index order (bitwise
- * reproducible): it sorts each element's particles by index (O(m log^2 m)
- * for m particles in an element), computes every particle's source into a
+ * reproducible): it sorts each element's particles by index (O(m^2) for
+ * m <= 128 particles in an element, O(m log^2 m) above), computes every particle's source into a
  * library-owned device buffer of 36 bytes per particle (grown on demand,
  * released by pt_destroy), then reduces per element.  Other mode bits: PT_ERR_ARG. */
 pt_status pt_deposit(pt_ctx* ctx, const pt_particles* p, int32_t mode, float* S_dev);

@@ -936,8 +936,15 @@ static pt_status ensure_scratch(pt_ctx* c, int64_t n) {
   return PT_OK;
 }
 
-static int push_block(pt_ctx* c) { return c->cfg.block > 0 ? c->cfg.block : 128; }
-// the push kernel is compiled for blocks of at most 128 threads
+// Threads per block of the resident kernel (compiled for at most 128).  Below
+// 2^16 particles single warps spread over more SMs (10 steps of 1000 / 16000
+// particles, NGeo 3, N 5: 606 / 507 us with 32 against 939 / 561 with 128; FP64
+// the same way by 2-15 %), above it 128 is up to 4 % better; the learned start
+// shares its weights in the block.
+static int push_block(pt_ctx* c, int64_t n = (int64_t)1 << 16) {
+  if (c->cfg.block > 0) return c->cfg.block;
+  return n < ((int64_t)1 << 16) && c->cfg.guess != PT_GUESS_MLP ? 32 : 128;
+}
 
 static int grid_for(pt_ctx* c, int64_t n, int block, int occ) {
   int64_t want = (n + block - 1) / block;
@@ -1045,13 +1052,22 @@ static cudaEvent_t take_event(pt_ctx* c, int kind = 0) {
   return e;
 }
 
-// particles from which PT_SCHEDULE_AUTO takes the staged schedule
-static const int64_t kStagedMin = (int64_t)1 << 18;
+// Particles from which PT_SCHEDULE_AUTO takes the staged schedule.  A stage of
+// the staged schedule pays about 60 us for the latency of its list kernels, the
+// resident one nothing; its kernels then run at twice the occupancy.  us per
+// call, resident / staged, 3 steps: NGeo 2, N 5 on 32^3: 1349 / 2492 at 2.5e5
+// particles, 2416 / 3319 at 5e5, 4387 / 4210 at 10^6; NGeo 4, N 6 on 20^3: 2332 /
+// 3124, 4433 / 5055 and 8445 / 7935; FP64, NGeo 2, N 5 on 24^3: 11978 / 14549 and
+// 22708 / 23817.  Where many particles meet walls the resident kernel's warps wait
+// for the FP64 intersections (7e5, NGeo 4, N 6, falling onto a wall: 5.1 ms against
+// 4.6), which puts the line at 2^19.  The learned start's tensor-core kernel exists
+// in the staged schedule only, which is ahead earlier with it.
+static const int64_t kStagedMin = (int64_t)1 << 19, kStagedMinMlp = (int64_t)1 << 18;
 
 static bool use_staged(const pt_ctx* c, int64_t n) {
   if (c->cfg.schedule == PT_SCHEDULE_STAGED) return true;
   if (c->cfg.schedule == PT_SCHEDULE_RESIDENT) return false;
-  return n >= kStagedMin;
+  return n >= (c->cfg.guess == PT_GUESS_MLP ? kStagedMinMlp : kStagedMin);
 }
 
 // Carves the staged schedule's state buffers for n particles out of one
@@ -1238,7 +1254,7 @@ pt_status pt_push_impl(pt_ctx* c, const pt_particles* p, int32_t nsteps, double 
     if (s) return s;
     const bool f64 = c->cfg.precision == PT_FP64;
     const int np = c->N + 1;
-    const int block = push_block(c);
+    const int block = push_block(c, n);
     int occ = max_active_push(c->g, f64, np, block);
     int grid = grid_for(c, n, block, occ);
     PushArgs a;
