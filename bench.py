@@ -176,12 +176,10 @@ def make_workload(args, device, seed, precision):
                             seed=seed, device=device, precision=precision)
 
 
-# DRAM bytes per particle-stage of the stage kernel k_stage_f32 (learned start),
-# from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum of one
-# launch on the 32^3, 10^6-particle channel, divided by its 10^6 particles;
-# profiles/); the traffic is per particle, so it scales with the particles of
-# a launch.  None while the kernel differs from the captured one.
-TRAFFIC_BYTES_PER_PARTICLE_STAGE = (235.257088e6 + 48.194816e6) / 1e6
+# DRAM bytes per particle-stage of the benched stage kernel, from an ncu capture
+# (dram__bytes_read.sum + dram__bytes_write.sum of one launch divided by its
+# particles).  None while the kernel has not been captured in this configuration.
+TRAFFIC_BYTES_PER_PARTICLE_STAGE = None
 
 
 def algorithmic_flops_per_particle_stage(G=4, NP=6, ntri=2, it_full=2.0, it_resid=2.0):
@@ -571,7 +569,7 @@ def main():
     flops_stage = algorithmic_flops_per_particle_stage(G=4, NP=wl.N + 1, ntri=2, it_full=it32,
                                                        it_resid=it64)
     if staged:
-        kname = "k_stage_f32<G=4,NP=6,%s>" % ("learned start" if guess else "trilinear start")
+        kname = "k_stage_sm_f32<G=4,NP=6,%s>" % ("learned start" if guess else "trilinear start")
         k_ms, k_n = kinds[1]
         flops_launch = flops_stage * P
     else:
