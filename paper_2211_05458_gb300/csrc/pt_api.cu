@@ -1084,12 +1084,12 @@ static pt_status stage_args(pt_ctx* c, int64_t n, StageArgs& a) {
   bytes += al((f64 ? 24 : 24) * nn);                  // xe
   bytes += f64 ? 0 : al(12 * nn);                     // guess
   bytes += (f64 ? 4 : 5) * al(4 * nn) + 256;          // e, hits, st, list(s), counters
-  if (c->state_cap < n || !c->d_state) {
+  if (c->state_cap < bytes || !c->d_state) {
     if (c->d_state) cudaFree(c->d_state);
     c->d_state = nullptr;
     c->state_cap = 0;
     CK(cudaMalloc(&c->d_state, bytes));
-    c->state_cap = n;
+    c->state_cap = bytes;
   }
   char* b = (char*)c->d_state;
   auto take = [&](size_t sz) {

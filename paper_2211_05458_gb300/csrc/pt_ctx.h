@@ -68,7 +68,7 @@ struct pt_ctx {
   pt_batch_plan* batch = nullptr;
   // particle state of the staged schedule (sorted order), grown on demand
   void* d_state = nullptr;
-  int64_t state_cap = 0;
+  size_t state_cap = 0;  // bytes (a particle takes more of them in FP64 mode)
   // pt_push_stage: the next stage expected (0: none open), the particles and
   // time step of the open sequence
   int stage_next = 0;

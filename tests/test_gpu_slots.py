@@ -48,3 +48,22 @@ def test_slots_equal_resident(ngeo, N, P, mlp):
     for k in ("x", "v", "elem", "hits", "status"):
         assert np.array_equal(a[k], b[k]), k
     assert sa["particle_steps"] == sb["particle_steps"] and sa["crossings"] == sb["crossings"]
+
+
+def test_state_buffer_follows_the_precision():
+    """A context whose precision is switched after a staged push allocates the
+    larger FP64 state: the result is a fresh FP64 context's."""
+    wl = W.curved_channel((4, 4, 4), 2, 3, P=3001, nsteps=3, dt=2e-3)
+    out = []
+    for switch in (True, False):
+        ctx = H.gpu_context(wl, "fp32" if switch else "fp64", schedule=pt.SCHEDULE_STAGED)
+        if switch:
+            ctx.push(H.gpu_particles(wl, ctx), 1, wl.dt)
+            ctx.set_config(precision=pt.FP64)
+            ctx.set_fluid(wl.N, wl.node_type, wl.U.to("cuda", torch.float64).contiguous())
+        parts = H.gpu_particles(wl, ctx)
+        ctx.push(parts, wl.nsteps, wl.dt)
+        out.append(H.gpu_result(parts))
+        ctx.close()
+    for k in ("x", "v", "elem", "hits", "status"):
+        assert np.array_equal(out[0][k], out[1][k]), k
