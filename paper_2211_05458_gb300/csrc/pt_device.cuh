@@ -1360,25 +1360,31 @@ __device__ __noinline__ void mortar_enter(const DevMesh& m, const DevConsts& k, 
 // Bound on how far xi(x + dx) can be from xi(x) + D, D = Ji dx, along the
 // straight segment dx: with the second derivatives of chi_r bounded by S_r
 // (DevMesh::curv) and K_d = sum_j |Ji_dj| S_j / 2, |xi - xi_lin|_d <= 2 K_d |D|^2
-// while K |D| <= 1/8 (else the bound is not used: returns false).  marg[d] is
-// that bound plus the distance band_x in reference units plus 1e-5 for the FP32
-// rounding of xi and Ji, curv the largest of the curvature parts.
+// while K |D| <= 1/8 (else the bound is not used: returns false).  D_d is a sum of
+// products that may cancel (a displacement along the long side of a thin element
+// that is not aligned with the axes), so its FP32 rounding scales with
+// sum_j |Ji_dj| |dx_j|: 2e-6 of that, some 30 roundings, for the Jacobian's Horner
+// sums, its inverse and the product.  bend is the largest of the curvature parts
+// and roundings, marg[d] their sum plus the distance band_x in reference units
+// plus 1e-5 for the FP32 rounding of xi.
 __device__ __forceinline__ bool xi_margin(const DevMesh& m, int e, const float* Ji,
                                           const float* dx, float bx, float* D, float* marg,
-                                          float& curv) {
+                                          float& bend) {
   const float4 S = __ldg(reinterpret_cast<const float4*>(m.curv) + e);
   matvec3(Ji, dx, D);
   const float a = tmax3(D[0], D[1], D[2]);
-  const float c[3] = {S.x * a * a, S.y * a * a, S.z * a * a};
-  curv = 0.f;
+  const float c[3] = {fmaf(2e-6f, fabsf(dx[0]), S.x * a * a),
+                      fmaf(2e-6f, fabsf(dx[1]), S.y * a * a),
+                      fmaf(2e-6f, fabsf(dx[2]), S.z * a * a)};
+  bend = 0.f;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float j0 = fabsf(Ji[3 * d]), j1 = fabsf(Ji[3 * d + 1]), j2 = fabsf(Ji[3 * d + 2]);
     const float q = j0 * c[0] + j1 * c[1] + j2 * c[2];
-    curv = fmaxf(curv, q);
+    bend = fmaxf(bend, q);
     marg[d] = q + (j0 + j1 + j2) * bx + 1e-5f;
   }
-  return curv <= 0.25f * a;
+  return bend <= 0.25f * a;
 }
 
 // True only if the stage segment from xi (inside element e) along dx cannot come
@@ -1389,8 +1395,8 @@ __device__ __forceinline__ bool xi_margin(const DevMesh& m, int e, const float* 
 // instead of 192.
 __device__ __forceinline__ bool stays_inside(const DevMesh& m, int e, const float* xi,
                                              const float* Ji, const float* dx, float bx) {
-  float D[3], marg[3], curv;
-  bool in = xi_margin(m, e, Ji, dx, bx, D, marg, curv);
+  float D[3], marg[3], bend;
+  bool in = xi_margin(m, e, Ji, dx, bx, D, marg, bend);
 #pragma unroll
   for (int d = 0; d < 3; ++d)
     in = in && fmaxf(fabsf(xi[d]), fabsf(xi[d] + D[d])) <= 1.f - marg[d];
@@ -1466,12 +1472,12 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
   while (true) {
     const float xf[3] = {x[0].hi, x[1].hi, x[2].hi};
     const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
-    float g[3], Ji[9], D[3], marg[3], curv;
+    float g[3], Ji[9], D[3], marg[3], bend;
     df zd[3];
     trilinear_guess(m, e, xf, g);
     bool jok;
     if (!newton_df<G>(m, k, e, x, g, zd, it32, it64, Ji, jok) || !jok) return false;
-    if (!xi_margin(m, e, Ji, dx, bx, D, marg, curv)) return false;
+    if (!xi_margin(m, e, Ji, dx, bx, D, marg, bend)) return false;
     unsigned faces = 0u;
     bool in = true;
 #pragma unroll
@@ -1493,7 +1499,7 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
       const float zq = q == 0 ? zd[0].hi : (q == 1 ? zd[1].hi : zd[2].hi);
       // the path (and band_x beyond its ends) is monotone across the face, so
       // that it meets the face once: slope Dq against the bend of the bound
-      if (!(fabsf(Dq) > fmaxf(2.f * ext * curv, 1e-2f * tmax3(D[0], D[1], D[2])))) return false;
+      if (!(fabsf(Dq) > fmaxf(2.f * ext * bend, 1e-2f * tmax3(D[0], D[1], D[2])))) return false;
       const float u = (zq - w) / Dq;  // 1 - tau at the face
       if (!(fabsf(u) < 4.f * ext)) continue;
       float s = q == 0 ? zd[1].hi - u * D[1] : zd[0].hi - u * D[0];
