@@ -1406,12 +1406,13 @@ __device__ __forceinline__ bool stays_inside(const DevMesh& m, int e, const floa
 // One Newton step d on F(s, t, alpha) = chi(s, t on face f) - (x + alpha td) = 0
 // from the Jacobian in FP32 and the double-float residual of the inverse map
 // (error ~1e-14 of the element); x a double-float offset, td the unit
-// direction.  cosr: the cosine between the ray and the face normal there.
+// direction.  cosr: the cosine between the ray and the face normal there; lat:
+// the largest change of s or t per unit of length of the right-hand side.
 // False if the Jacobian is singular.
 template <int G>
 __device__ __forceinline__ bool face_step(const DevMesh& m, int e, int tm, int f, const df* x,
                                           const float* td, float s, float t, float al, float* d,
-                                          float& cosr) {
+                                          float& cosr, float& lat) {
   const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
   const int q = f >> 1;
   const float w = (f & 1) ? 1.f : -1.f;
@@ -1433,6 +1434,8 @@ __device__ __forceinline__ bool face_step(const DevMesh& m, int e, int tm, int f
   resid_df<G>(Mh, m.monolo + (size_t)e * 3 * Mono<G>::CS, xi, tm, xa, F);
   // row 3 of Ai is -n / (n . td), n the face normal p_s x p_t
   cosr = 1.f / sqrtf(Ai[6] * Ai[6] + Ai[7] * Ai[7] + Ai[8] * Ai[8]);
+  lat = fmaxf(fabsf(Ai[0]) + fabsf(Ai[1]) + fabsf(Ai[2]),
+              fabsf(Ai[3]) + fabsf(Ai[4]) + fabsf(Ai[5]));
   matvec3(Ai, F, d);
   return true;
 }
@@ -1442,10 +1445,15 @@ __device__ __forceinline__ bool face_step(const DevMesh& m, int e, int tm, int f
 // current element the end point's xi is found by the inverse map, and the
 // segment's path is xi - (1 - tau) D up to the bound of xi_margin.  Only faces
 // that the path can come to within the bands are intersected: the linear path
-// gives the start, two Newton steps with the double-float residual leave alpha
-// good to ~1e-13 of the element over the cosine to the face, and acceptance
-// and the near-face bands are decided with margins (tb, 2e-6 in s and t) four
-// orders above that.  The smallest accepted alpha wins; an internal or
+// gives the start, two Newton steps with the double-float residual follow.  The
+// direction, the length and alpha itself are single FP32 numbers, so the crossing
+// is good to a few roundings (6e-8) of the length L, whatever the residual is:
+// acceptance and the near-face bands are decided with the margins tb on alpha,
+// 1e-6 (L + band_x) plus 1e-8 of the element over the cosine to the face, and ms
+// on s and t, 2e-6 plus 1e-6 (L + band_x) in reference units; an end that is not
+// inside by a rounding is not decided here either.  (With 1e-8 of L, 3 % of the
+// ends up to 1e-7 beyond a wall were taken as inside at L from 0.2 elements on.)
+// The smallest accepted alpha wins; an internal or
 // periodic face leads to the next element, the position is the segment's end.
 // A wall, open or mortar face that is hit, a path nearly parallel to a face it
 // may reach, a quantity within the margin of its threshold and two crossings
@@ -1457,7 +1465,7 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
                                           TrackCounters& tc) {
   int e = e_io, cross = 0, fin = -1;
   unsigned bits = 0u;
-  float dx[3], td[3], a0 = 0.f;
+  float dx[3], td[3], a0 = 0.f, a0tb = 0.f;
   df x[3] = {xe[0], xe[1], xe[2]};      // the segment's ends in the current element's frame
   df x0[3] = {xd[0], xd[1], xd[2]};
   double xg[3] = {0.0, 0.0, 0.0}, xs[3] = {0.0, 0.0, 0.0};  // global, once it has crossed
@@ -1485,7 +1493,7 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
       const float z1 = zd[d].hi, z0 = z1 - D[d];
       if (fmaxf(z0, z1) > 1.f - marg[d]) faces |= 2u << (2 * d);
       if (fminf(z0, z1) < -1.f + marg[d]) faces |= 1u << (2 * d);
-      in = in && fabsf(z1) <= 1.f;
+      in = in && fabsf(z1) < 1.f;
     }
     if (fin >= 0) faces &= ~(1u << fin);
     int pf = -1;
@@ -1504,10 +1512,10 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
       if (!(fabsf(u) < 4.f * ext)) continue;
       float s = q == 0 ? zd[1].hi - u * D[1] : zd[0].hi - u * D[0];
       float t = q == 2 ? zd[1].hi - u * D[1] : zd[2].hi - u * D[2];
-      float al = L - u * L, d[3], cosr = 0.f;
+      float al = L - u * L, d[3], cosr = 0.f, lat = 0.f;
 #pragma unroll 1
       for (int it = 0; it < 2; ++it) {
-        if (!face_step<G>(m, e, tm, f, x0, td, s, t, al, d, cosr)) return false;
+        if (!face_step<G>(m, e, tm, f, x0, td, s, t, al, d, cosr, lat)) return false;
         s -= d[0];
         t -= d[1];
         al -= d[2];
@@ -1515,11 +1523,12 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
       if (!(cosr > 1e-3f) || !(fabsf(d[0]) < 1e-5f && fabsf(d[1]) < 1e-5f && fabsf(d[2]) < 1e-4f * (L + bx)))
         return false;
       const float Rmax = __ldg(m.slab + 48 * (size_t)e + 5);
-      const float mm = fmaxf(fabsf(s), fabsf(t)), tb = 1e-8f * (Rmax + L) / cosr;
+      const float el = 1e-6f * (L + bx), mm = fmaxf(fabsf(s), fabsf(t));
+      const float ms = 2e-6f + el * lat, tb = (1e-8f * Rmax + el) / cosr, ta = tb + a0tb;
       const float om = mm - 1.f, da = al - a0, dL = L - al;
-      if (om > br + 2e-6f || da < -bx - tb || dL < -bx - tb) continue;
-      if (fabsf(om) <= 2e-6f || fabsf(fabsf(om) - br) <= 2e-6f || fabsf(da) <= tb ||
-          fabsf(dL) <= tb || fabsf(fabsf(da) - bx) <= tb || fabsf(fabsf(dL) - bx) <= tb)
+      if (om > br + ms || da < -bx - ta || dL < -bx - tb) continue;
+      if (fabsf(om) <= ms || fabsf(fabsf(om) - br) <= ms || fabsf(da) <= ta ||
+          fabsf(dL) <= tb || fabsf(fabsf(da) - bx) <= ta || fabsf(fabsf(dL) - bx) <= tb)
         return false;
       const int bc = finfo_bc(__ldg(m.finfo + 6 * (size_t)e + f));
       if (fabsf(om) < br || fabsf(da) < bx || fabsf(dL) < bx)
@@ -1561,6 +1570,7 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
     fin = finfo_nf(info);
     e = __ldg(m.fnbr + 6 * (size_t)e + pf);
     a0 = pal;
+    a0tb = ptb;
     const double* cn = m.ce + 3 * (size_t)e;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {

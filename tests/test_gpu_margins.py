@@ -1,8 +1,9 @@
 """Decisions that the FP32 mode takes in single precision, at the ends of the
 ranges that their margins have to cover: long stage displacements in thin
-elements that are not aligned with the axes.  The drag is masked, so that a
-particle moves on a straight line and the stage displacements are known
-beforehand."""
+elements that are not aligned with the axes and ends a rounding beyond a wall.
+Against the FP64 oracle
+or the exact path, particle by particle.  The drag is masked, so that a particle moves on a
+straight line and the stage displacements are known beforehand."""
 import numpy as np
 import pytest
 import torch
@@ -75,3 +76,33 @@ def test_long_displacements_in_thin_rotated_elements(aspect, length, ngeo, sched
     own = np.stack([e % n[0], e // n[0] % n[1], e // (n[0] * n[1])], 1)
     z = 2.0 * ((g["x"] @ R) / h - own) - 1.0
     assert np.abs(z).max() <= 1.0 + 1e-6  # lost_tol
+
+
+@pytest.mark.parametrize("schedule", SCHEDULES)
+@pytest.mark.parametrize("ngeo", [1, 2])
+@pytest.mark.parametrize("length", [0.05, 0.2, 0.4, 0.9])
+def test_ends_a_rounding_beyond_a_wall(length, ngeo, schedule):
+    """Unit cubes, the first stage ending 0 to 1e-7 beyond a wall: it is
+    reflected there or, if the end is taken as inside, at the next stage's
+    start, and never lost."""
+    P = 20_000
+    mesh = W.box_mesh((3, 3, 3), (0.0, 0.0, 0.0), (3.0, 3.0, 3.0), ngeo, (False,) * 3)
+    rng = np.random.default_rng(int(100 * length) + ngeo)
+    jk = rng.integers(0, 3, (P, 2))
+    elem = 2 + 3 * (jk[:, 0] + 3 * jk[:, 1])
+    cos = rng.uniform(0.5, 1.0, P)
+    phi = rng.uniform(0.0, 2.0 * np.pi, P)
+    t = np.sqrt(1.0 - cos * cos)
+    dx = length * np.stack([cos, t * np.cos(phi), t * np.sin(phi)], 1)
+    v = (dx / (B0 * DT)).astype(np.float32)
+    # the displacement as the FP32 mode forms it
+    d1 = (np.float32(B0) * (np.float32(DT) * v[:, 0])).astype(np.float64)
+    x = np.stack([3.0 + rng.uniform(0.0, 1e-7, P) - d1, jk[:, 0] + rng.uniform(0.05, 0.95, P),
+                  jk[:, 1] + rng.uniform(0.05, 0.95, P)], 1)
+    wl = _workload(mesh, x, elem, v)
+    o = H.run_oracle(wl, mask=(0.0, 0.0, 0.0))
+    assert _frozen(o) == 0 and int((o["hits"] > 0).sum()) == P
+    g = _push(wl, schedule=schedule)
+    assert _frozen(g) == 0
+    assert np.array_equal(g["hits"], o["hits"])
+    assert np.abs(g["x"] - o["x"]).max() <= 30 * 6e-8 * length / B0
