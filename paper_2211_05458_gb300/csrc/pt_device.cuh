@@ -324,10 +324,11 @@ __device__ __forceinline__ bool newton_f64(const DevMesh& m, const DevConsts& k,
 
 // Mixed-precision Newton on a double-float local position xd (relative to the
 // element centre): FP32 iterations (chi and J in FP32) until the step is below
-// 1e-5, then double-float residuals with the last FP32 inverse Jacobian until
+// 1e-5 (after eight of them 1e-3 will do: in thin elements rounding keeps it above
+// 1e-5; sixteen that do not get there count as failed), then double-float residuals with the last FP32 inverse Jacobian until
 // the step is below newton_tol.  Returns the double-float xi in zd and, unless
 // the (out-of-line) fallback of a full FP64 Newton was taken (jok false), the
-// inverse Jacobian at xi to ~1e-5 in Ji.
+// inverse Jacobian of a point within about 1e-3 of xi (1e-5 as a rule) in Ji.
 // GEN: the element's coefficients (high, low parts) may be in shared memory,
 // at Mh and Ml.
 template <int G, bool GEN = false>
@@ -344,7 +345,7 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
   bool have = false;
   jok = true;
   #pragma unroll 1
-  for (int it = 0; it < 8; ++it) {
+  for (int it = 0;; ++it) {
     float chi[3], J[9], r[3], d[3];
     map_j32<G, GEN>(Mh, z, tm, chi, J);
     if (!inv3(J, Ji)) break;
@@ -359,7 +360,11 @@ __device__ __forceinline__ bool newton_df(const DevMesh& m, const DevConsts& k, 
       have = false;
       break;
     }
-    if (tmax3(d[0], d[1], d[2]) < PT_NEWTON_SWITCH) break;
+    if (tmax3(d[0], d[1], d[2]) < (it < 7 ? PT_NEWTON_SWITCH : 1e-3f)) break;
+    if (it == 15) {
+      have = false;
+      break;
+    }
   }
   if (have) {
 #pragma unroll
@@ -1358,31 +1363,36 @@ __device__ __noinline__ void mortar_enter(const DevMesh& m, const DevConsts& k, 
 }
 
 // Bound on how far xi(x + dx) can be from xi(x) + D, D = Ji dx, along the
-// straight segment dx: with the second derivatives of chi_r bounded by S_r
-// (DevMesh::curv) and K_d = sum_j |Ji_dj| S_j / 2, |xi - xi_lin|_d <= 2 K_d |D|^2
-// while K |D| <= 1/8 (else the bound is not used: returns false).  D_d is a sum of
-// products that may cancel (a displacement along the long side of a thin element
-// that is not aligned with the axes), so its FP32 rounding scales with
-// sum_j |Ji_dj| |dx_j|: 2e-6 of that, some 30 roundings, for the Jacobian's Horner
-// sums, its inverse and the product.  bend is the largest of the curvature parts
-// and roundings, marg[d] their sum plus the distance band_x in reference units
-// plus 1e-5 for the FP32 rounding of xi.
+// straight segment dx: with the second derivatives of chi_r bounded by S_r and
+// K_d = sum_j |Ji_dj| S_j / 2, |xi - xi_lin|_d <= 2 K_d |D|^2 while K |D| <= 1/8
+// (else the bound is not used: returns false).  |D| is taken larger by what the
+// path is extended by the distance band_x at its ends and by 1e-3, how far from xi
+// Ji may have been evaluated (newton_df).  S_r = grow DevMesh::curv, which holds
+// for |xi| <= 1.1; the caller says by grow how far the path goes beyond (1 if it
+// does not).  D_d is a sum of products that may cancel (a displacement along the
+// long side of a thin element that is not aligned with the axes), so its FP32
+// rounding scales with sum_j |Ji_dj| |dx_j|: 2e-6 of that, some 30 roundings, for
+// the Jacobian's Horner sums, its inverse and the product.  bend is the largest of
+// the curvature parts and roundings, marg[d] their sum plus band_x in reference
+// units plus 1e-5 for the FP32 rounding of xi.
 __device__ __forceinline__ bool xi_margin(const DevMesh& m, int e, const float* Ji,
-                                          const float* dx, float bx, float* D, float* marg,
-                                          float& bend) {
+                                          const float* dx, const float* D, float bx, float grow,
+                                          float* marg, float& bend) {
   const float4 S = __ldg(reinterpret_cast<const float4*>(m.curv) + e);
-  matvec3(Ji, dx, D);
-  const float a = tmax3(D[0], D[1], D[2]);
-  const float c[3] = {fmaf(2e-6f, fabsf(dx[0]), S.x * a * a),
-                      fmaf(2e-6f, fabsf(dx[1]), S.y * a * a),
-                      fmaf(2e-6f, fabsf(dx[2]), S.z * a * a)};
+  float b[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    b[d] = (fabsf(Ji[3 * d]) + fabsf(Ji[3 * d + 1]) + fabsf(Ji[3 * d + 2])) * bx;
+  const float a = tmax3(D[0], D[1], D[2]) + tmax3(b[0], b[1], b[2]) + 1e-3f, a2 = grow * a * a;
+  const float c[3] = {fmaf(2e-6f, fabsf(dx[0]), S.x * a2), fmaf(2e-6f, fabsf(dx[1]), S.y * a2),
+                      fmaf(2e-6f, fabsf(dx[2]), S.z * a2)};
   bend = 0.f;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float j0 = fabsf(Ji[3 * d]), j1 = fabsf(Ji[3 * d + 1]), j2 = fabsf(Ji[3 * d + 2]);
-    const float q = j0 * c[0] + j1 * c[1] + j2 * c[2];
+    const float q =
+        fabsf(Ji[3 * d]) * c[0] + fabsf(Ji[3 * d + 1]) * c[1] + fabsf(Ji[3 * d + 2]) * c[2];
     bend = fmaxf(bend, q);
-    marg[d] = q + (j0 + j1 + j2) * bx + 1e-5f;
+    marg[d] = q + b[d] + 1e-5f;
   }
   return bend <= 0.25f * a;
 }
@@ -1396,7 +1406,8 @@ __device__ __forceinline__ bool xi_margin(const DevMesh& m, int e, const float* 
 __device__ __forceinline__ bool stays_inside(const DevMesh& m, int e, const float* xi,
                                              const float* Ji, const float* dx, float bx) {
   float D[3], marg[3], bend;
-  bool in = xi_margin(m, e, Ji, dx, bx, D, marg, bend);
+  matvec3(Ji, dx, D);
+  bool in = xi_margin(m, e, Ji, dx, D, bx, 1.f, marg, bend);
 #pragma unroll
   for (int d = 0; d < 3; ++d)
     in = in && fmaxf(fabsf(xi[d]), fabsf(xi[d] + D[d])) <= 1.f - marg[d];
@@ -1485,7 +1496,23 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
     trilinear_guess(m, e, xf, g);
     bool jok;
     if (!newton_df<G>(m, k, e, x, g, zd, it32, it64, Ji, jok) || !jok) return false;
-    if (!xi_margin(m, e, Ji, dx, bx, D, marg, bend)) return false;
+    matvec3(Ji, dx, D);
+    // The segment leaves the element, so the path may reach far beyond the range
+    // that the curvature bound holds for: from its end back to where it came in,
+    // and 0.1 to the sides, which the margins may not exceed.  There a second
+    // derivative's terms of total degree n <= 3 (G - 1) are at most (z / 1.1)^(n - 2) /
+    // 1.1^2 times the bound's.
+    const float back = 1.f - a0 / L;
+    float zr = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      zr = fmaxf(zr, fmaxf(fabsf(zd[d].hi), fabsf(zd[d].hi - back * D[d])));
+    const float zq1 = (zr + 0.1f) * (1.f / 1.1f);
+    float grow = 1.f / 1.21f;
+#pragma unroll
+    for (int p = 0; p < 3 * G - 5; ++p) grow *= zq1;
+    if (!xi_margin(m, e, Ji, dx, D, bx, fmaxf(grow, 1.f), marg, bend)) return false;
+    if (!(tmax3(marg[0], marg[1], marg[2]) <= 0.1f)) return false;
     unsigned faces = 0u;
     bool in = true;
 #pragma unroll

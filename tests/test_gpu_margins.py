@@ -1,7 +1,7 @@
 """Decisions that the FP32 mode takes in single precision, at the ends of the
 ranges that their margins have to cover: long stage displacements in thin
-elements that are not aligned with the axes and ends a rounding beyond a wall.
-Against the FP64 oracle
+elements that are not aligned with the axes, ends a rounding beyond a wall, and
+segments that leave an element by more than its size.  Against the FP64 oracle
 or the exact path, particle by particle.  The drag is masked, so that a particle moves on a
 straight line and the stage displacements are known beforehand."""
 import numpy as np
@@ -106,3 +106,65 @@ def test_ends_a_rounding_beyond_a_wall(length, ngeo, schedule):
     assert _frozen(g) == 0
     assert np.array_equal(g["hits"], o["hits"])
     assert np.abs(g["x"] - o["x"]).max() <= 30 * 6e-8 * length / B0
+
+
+@pytest.mark.parametrize("schedule", SCHEDULES)
+@pytest.mark.parametrize("ngeo,c,reach", [(4, 0.0035, 2.5), (4, 0.004, 2.4), (4, 0.003, 2.7),
+                                          (4, 0.01, 1.5), (3, 0.01, 2.5), (2, 0.02, 2.0)])
+def test_segments_that_leave_the_element_far_behind(ngeo, c, reach, schedule):
+    """Elements stretched along x by xi + c (xi^p - 1 or xi), first stages from
+    within band_x of the wall at x = 0 to xi = reach in the first element's
+    extended map, where its curvature is far above that inside: the wall that
+    the segment starts at still counts as met (PT_ST_NEAR_WALL)."""
+    P, nx, band = 2000, 24, 1e-3
+    odd = ngeo % 2 == 1
+    g1 = (lambda s: s + c * (s ** ngeo - s)) if odd else (lambda s: s + c * (s ** ngeo - 1.0))
+    mesh = W.box_mesh((nx, 2, 2), (0.0, 0.0, 0.0), (float(nx), 2.0, 2.0), ngeo, (False,) * 3)
+    s = np.linspace(-1.0, 1.0, ngeo + 1)
+    i = np.arange(mesh.nelem) % nx
+    X = mesh.xgeo.reshape(mesh.nelem, -1, ngeo + 1, 3)  # (xi1 fastest)
+    X[..., 0] = i[:, None, None] + 0.5 * (1.0 + g1(s))[None, None, :]
+    rng = np.random.default_rng(ngeo)
+    jk = rng.integers(0, 2, (P, 2))
+    elem = nx * (jk[:, 0] + 2 * jk[:, 1])
+    x = np.stack([rng.uniform(0.1, 0.8, P) * band, jk[:, 0] + rng.uniform(0.4, 0.6, P),
+                  jk[:, 1] + rng.uniform(0.4, 0.6, P)], 1)
+    dx = np.zeros((P, 3))
+    dx[:, 0] = 0.5 * (1.0 + g1(reach)) - x[:, 0]
+    wl = _workload(mesh, x, elem, dx / (B0 * DT))
+    o = H.run_oracle(wl, band_x=band, mask=(0.0, 0.0, 0.0))
+    assert _frozen(o) == 0 and bool((o["status"] & oracle.ST_NEAR_WALL).all())
+    g = _push(wl, schedule=schedule, band_x=band)
+    assert _frozen(g) == 0 and np.array_equal(g["elem"], o["elem"])
+    missed = (g["status"] & oracle.ST_NEAR_WALL) == 0
+    assert not missed.any(), int(missed.sum())
+
+
+@pytest.mark.parametrize("ngeo", [2, 3, 4])
+def test_large_steps_between_curved_walls(ngeo):
+    """Stage displacements up to about an element between curved walls: owners,
+    wall hits, states and positions are those of the FP64 mode, which intersects
+    every face in FP64."""
+    mesh = W.channel_mesh((6, 5, 4), ngeo, amp=0.1, curved_walls=True)
+    P = 600
+    wl = W.curved_channel((6, 5, 4), ngeo, 3, P=P, nsteps=2, dt=0.15, seed=ngeo)
+    wl.mesh = mesh
+    wl.U, _ = W.fluid_channel(mesh, 3, 0, seed=0)
+    wl.x, wl.elem = W.seed_particles(mesh, P, seed=ngeo)
+    rng = np.random.default_rng(ngeo)
+    wl.v = torch.as_tensor(rng.normal(size=(P, 3)) * np.array([6.0, 3.0, 4.0]))
+    wl.v = wl.v.float().double()
+    wl.d = torch.full((P,), 2e-2, dtype=torch.float64)  # Stokes number 2200: nearly straight
+    band = dict(band_ref=2e-4, band_x=4e-5)
+    out = []
+    for precision in ("fp32", "fp64"):
+        ctx = H.gpu_context(wl, precision, **band)
+        parts = H.gpu_particles(wl, ctx)
+        ctx.push(parts, wl.nsteps, wl.dt)
+        torch.cuda.synchronize()
+        out.append(H.gpu_result(parts))
+        ctx.close()
+    ref = out[1]
+    assert int(ref["hits"].sum()) > P // 4
+    ref["_orc"], ref["_params"] = H.make_oracle(wl), H.oracle_params(wl, **band)
+    H.compare(out[0], ref, 2e-5, min_checked=0.85)
