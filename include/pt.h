@@ -232,7 +232,9 @@ void pt_config_default(pt_config* cfg);
 pt_status pt_init_mesh(pt_ctx** ctx, const pt_mesh_desc* mesh, const pt_config* cfg,
                        void* stream);
 
-/* Replaces the configuration (same rules as at init). */
+/* Replaces the configuration (same rules as at init; band_x is fixed at init,
+ * PT_ERR_ARG).  PT_ERR_STATE for another precision while a pt_push_stage
+ * sequence is open. */
 pt_status pt_set_config(pt_ctx* ctx, const pt_config* cfg);
 
 /* Registers the fluid state (Sec. 3.1, Eq. dgsem_interpolation): N in 1..7,

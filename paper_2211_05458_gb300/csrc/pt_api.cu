@@ -896,6 +896,10 @@ pt_status pt_set_config(pt_ctx* c, const pt_config* cfg) {
   }
   if (cfg->band_x != c->cfg.band_x)
     return fail(c, PT_ERR_ARG, "band_x is fixed at init (it sizes the face slabs)");
+  // the state that stage 0 filled is laid out by the precision
+  if (c->stage_next != 0 && cfg->precision != c->cfg.precision)
+    return fail(c, PT_ERR_STATE, "the precision is fixed while a pt_push_stage sequence is open "
+                "(stage %d expected)", c->stage_next);
   c->cfg = *cfg;
   return PT_OK;
 }
