@@ -265,61 +265,62 @@ __device__ __noinline__ bool newton64_cold(const double* M, const double* xl, do
 // confirm |dxi| < tol) evaluate the FP64 residual alone and keep the FP64
 // inverse Jacobian of that step, whose relative error is the step's size.  The
 // fixed point is the FP64 residual's zero, as with full Newton steps, which
-// took 3 to 4 evaluations of the FP64 map and Jacobian from the trilinear start
-// and remain the fallback.
+// took 3 to 4 evaluations of the FP64 map and Jacobian from the trilinear start.
+// Where the FP32 iterations do not settle in six, or the FP64 steps leave the
+// range, meet a singular Jacobian or take more than four, full Newton steps run
+// from the start that was given: whatever they converge from is found.
 template <int G>
 __device__ __forceinline__ bool newton_f64(const DevMesh& m, const DevConsts& k, int e,
                                            const double* xl, const float* guess, double* xi,
                                            int& it64) {
   const double* M = m.mono64 + (size_t)e * 3 * G * G * G;
+  bool settled = false;
   {
     const float* Mh = m.mono + (size_t)e * 3 * Mono<G>::CS;
     const int tm = G == 2 ? 7 : __ldg(m.tmask + e);
     const float xf[3] = {(float)xl[0], (float)xl[1], (float)xl[2]};
     float z[3] = {guess[0], guess[1], guess[2]};
-    bool ok = true;
 #pragma unroll 1
-    for (int it = 0; it < 6 && ok; ++it) {
+    for (int it = 0; it < 6; ++it) {
       float chi[3], J[9], Ji[9], r[3], d[3];
       map_j32<G>(Mh, z, tm, chi, J);
-      if (!inv3(J, Ji)) {
-        ok = false;
-        break;
-      }
+      if (!inv3(J, Ji)) break;
 #pragma unroll
       for (int q = 0; q < 3; ++q) r[q] = chi[q] - xf[q];
       matvec3(Ji, r, d);
 #pragma unroll
       for (int q = 0; q < 3; ++q) z[q] -= d[q];
-      ok = tmax3(z[0], z[1], z[2]) <= 4.f;
-      if (tmax3(d[0], d[1], d[2]) < PT_NEWTON_SWITCH) break;
+      if (!(tmax3(z[0], z[1], z[2]) <= 4.f)) break;
+      settled = tmax3(d[0], d[1], d[2]) < PT_NEWTON_SWITCH;
+      if (settled) break;
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) xi[q] = ok ? z[q] : guess[q];
+    for (int q = 0; q < 3; ++q) xi[q] = z[q];
   }
-  const int maxit = k.max_newton;
-  double chi[3], Ji[9], r[3], d[3];
-  {
-    double J[9];
+  double chi[3], J[9], Ji[9], r[3], d[3];
+  if (settled) {
     map64<G, true>(M, xi, chi, J);
-    if (!inv3(J, Ji)) return false;
+    settled = inv3(J, Ji);
   }
-  int it = 0;
+  if (settled) {
+    const int maxit = k.max_newton < 4 ? k.max_newton : 4;
+    int it = 0;
 #pragma unroll 1
-  while (true) {
+    while (true) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) r[q] = chi[q] - xl[q];
-    matvec3(Ji, r, d);
+      for (int q = 0; q < 3; ++q) r[q] = chi[q] - xl[q];
+      matvec3(Ji, r, d);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) xi[q] -= d[q];
-    ++it64;
-    ++it;
-    if (tmax3(d[0], d[1], d[2]) < k.newton_tol) return true;
-    if (!(tmax3(xi[0], xi[1], xi[2]) <= 4.0) || it >= maxit) return false;
-    if (it >= 4) break;
-    map64<G, false>(M, xi, chi, nullptr);
+      for (int q = 0; q < 3; ++q) xi[q] -= d[q];
+      ++it64;
+      if (tmax3(d[0], d[1], d[2]) < k.newton_tol) return true;
+      if (!(tmax3(xi[0], xi[1], xi[2]) <= 4.0) || ++it >= maxit) break;
+      map64<G, false>(M, xi, chi, nullptr);
+    }
   }
-  return newton64_cold<G>(M, xl, xi, k, maxit - it, it64);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) xi[q] = guess[q];
+  return newton64_cold<G>(M, xl, xi, k, k.max_newton, it64);
 }
 
 // Mixed-precision Newton on a double-float local position xd (relative to the
