@@ -1220,29 +1220,13 @@ struct TrackCounters {
   int cross, hits, slow;
 };
 
-// Conservative FP32 test: can the segment a -> b (element-local coordinates,
-// extended by the band) touch any face of element e?  Slab of face f:
+// Conservative FP32 test: which kind of face of element e can the segment a -> b
+// (element-local coordinates, extended by the band) touch: bit 0 some face (or a
+// long segment), bit 1 a wall or open face (or a long segment).  Slab of face f:
 // lo <= n.(P - ce) <= hi for every point of the face, margins (band plus
 // 4e-6 of the element radius, which covers the FP32 rounding of a and b while
-// they stay within 8 radii) included; longer segments take the exact path.
-__device__ __forceinline__ bool touches_any_slab(const DevMesh& m, int e, const float* a,
-                                                 const float* b) {
-  const float4* S = reinterpret_cast<const float4*>(m.slab + 48 * (size_t)e);
-  const float rlim = 8.f * __ldg(m.slab + 48 * (size_t)e + 5);
-  bool hit = !(fmaxf(fmaxf(fabsf(b[0]), fabsf(b[1])), fabsf(b[2])) <= rlim);
-#pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    float4 s0 = __ldg(S + 2 * f), s1 = __ldg(S + 2 * f + 1);
-    float pa = s0.x * a[0] + s0.y * a[1] + s0.z * a[2];
-    float pb = s0.x * b[0] + s0.y * b[1] + s0.z * b[2];
-    hit |= (fmaxf(pa, pb) >= s0.w) && (fminf(pa, pb) <= s1.x);
-  }
-  return hit;
-}
-
-// As touches_any_slab, with the kind of face: bit 0 some face (or a long
-// segment), bit 1 a wall or open face (or a long segment).  Slab word 7 flags
-// the wall and open faces.
+// they stay within 8 radii) included; longer segments take the exact path.  Slab
+// word 7 flags the wall and open faces.
 __device__ __forceinline__ int slab_touch(const DevMesh& m, int e, const float* a,
                                           const float* b) {
   const float4* S = reinterpret_cast<const float4*>(m.slab + 48 * (size_t)e);
@@ -1256,31 +1240,6 @@ __device__ __forceinline__ int slab_touch(const DevMesh& m, int e, const float* 
     if ((fmaxf(pa, pb) >= s0.w) && (fminf(pa, pb) <= s1.x)) t |= s1.w != 0.f ? 3 : 1;
   }
   return t;
-}
-
-// Tracks the stage segment x -> xe through the mesh.  The ray
-// x(alpha) = xs + alpha td, alpha in (a0, L] (Eq. parttrajectory) is tested
-// against every face of the current element except the entry face; the
-// smallest accepted alpha wins (lowest face index on ties).  Internal face:
-// continue in the neighbour on the same ray.  Periodic: same, translated.
-// Wall: restart at the hit point with the remaining length, mirroring the
-// direction, v, kx and kv by I - 2 n n^T (Sec. 2.4).  Open: stop there.
-template <int G, typename R, bool CLIP = false>
-__device__ __noinline__ void track_slow(const DevMesh& m, const DevConsts& k, int& e, double* x,
-                                        double* xe, R* v, R* kx, R* kv, int& hits, unsigned& st,
-                                        TrackCounters& tc);
-
-// a, b: segment ends relative to the element centre in FP32 (for the test only)
-template <int G, typename R>
-__device__ __forceinline__ void track(const DevMesh& m, const DevConsts& k, int& e, double* x,
-                                      double* xe, const float* a, const float* b, R* v, R* kx,
-                                      R* kv, int& hits, unsigned& st, TrackCounters& tc) {
-  if (!touches_any_slab(m, e, a, b)) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) x[r] = xe[r];
-    return;
-  }
-  track_slow<G, R>(m, k, e, x, xe, v, kx, kv, hits, st, tc);
 }
 
 // Big side of a mortar (Sec. 3.2.3): the crossing found on the big face is
@@ -1617,6 +1576,13 @@ __device__ __forceinline__ bool track_f32(const DevMesh& m, const DevConsts& k, 
   return true;
 }
 
+// Tracks the stage segment x -> xe through the mesh.  The ray
+// x(alpha) = xs + alpha td, alpha in (a0, L] (Eq. parttrajectory) is tested
+// against every face of the current element except the entry face; the
+// smallest accepted alpha wins (lowest face index on ties).  Internal face:
+// continue in the neighbour on the same ray.  Periodic: same, translated.
+// Wall: restart at the hit point with the remaining length, mirroring the
+// direction, v, kx and kv by I - 2 n n^T (Sec. 2.4).  Open: stop there.
 // CLIP: curved faces by Bezier clipping (a separate instantiation, so that the
 // default path carries none of its code)
 template <int G, typename R, bool CLIP>
