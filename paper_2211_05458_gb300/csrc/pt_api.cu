@@ -433,7 +433,8 @@ static cudaError_t launch_mono(pt_ctx* c) {
     default: k_mono<5><<<nb, 128, 0, c->stream>>>(c->d_xg64, c->d_tmask, c->nelem, V, c->d_mono, c->d_monolo, c->d_mono64, c->d_curv); break;
   }
   const cudaError_t err = cudaGetLastError();
-  return err ? err : cudaStreamSynchronize(c->stream);
+  const cudaError_t done = cudaStreamSynchronize(c->stream);
+  return err ? err : done;
 }
 
 static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
@@ -709,8 +710,14 @@ static pt_status upload_mesh(pt_ctx* c, const pt_mesh_desc* md) {
             {c->d_shift, shift.data(), shift.size() * 8},
             {c->d_mort, mort.data(), mort.size() * 4}};
   for (auto& q : cp) {
-    err = cudaMemcpy(q.d, q.h, q.b, cudaMemcpyHostToDevice);
-    if (err) return fail(nullptr, PT_ERR_CUDA, "cudaMemcpy: %s", cudaGetErrorString(err));
+    // in the order of the stream that k_mono and all later work run on: a plain
+    // cudaMemcpy may return before its transfer is done, and a non-blocking stream
+    // does not wait for it
+    err = cudaMemcpyAsync(q.d, q.h, q.b, cudaMemcpyHostToDevice, c->stream);
+    if (err) {
+      cudaStreamSynchronize(c->stream);  // the copies under way read this call's vectors
+      return fail(nullptr, PT_ERR_CUDA, "cudaMemcpyAsync: %s", cudaGetErrorString(err));
+    }
   }
   err = launch_mono(c);
   if (err) return fail(nullptr, PT_ERR_CUDA, "element map: %s", cudaGetErrorString(err));
@@ -1638,9 +1645,13 @@ static pt_status build_find_grid(pt_ctx* c) {
     if (err) return fail(c, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
     c->d_cell_elem = dmalloc<int>(c, std::max<size_t>(list.size(), 1), &err);
     if (err) return fail(c, PT_ERR_CUDA, "cudaMalloc: %s", cudaGetErrorString(err));
-    CK(cudaMemcpy(c->d_cell_start, start.data(), start.size() * 4, cudaMemcpyHostToDevice));
-    if (!list.empty())
-      CK(cudaMemcpy(c->d_cell_elem, list.data(), list.size() * 4, cudaMemcpyHostToDevice));
+    err = cudaMemcpyAsync(c->d_cell_start, start.data(), start.size() * 4, cudaMemcpyHostToDevice,
+                          c->stream);
+    if (!err && !list.empty())
+      err = cudaMemcpyAsync(c->d_cell_elem, list.data(), list.size() * 4, cudaMemcpyHostToDevice,
+                            c->stream);
+    const cudaError_t done = cudaStreamSynchronize(c->stream);  // start, list are local
+    CK(err ? err : done);
     for (int r = 0; r < 3; ++r) {
       c->grid_lo[r] = lo[r];
       c->grid_ih[r] = 1.0 / h;

@@ -365,8 +365,15 @@ extern "C" pt_status pt_push_batch(pt_ctx* const* ctxs, const pt_particles* part
       c0->err = "pt_push_batch: device allocation failed";
       return PT_ERR_CUDA;
     }
-    cudaMemcpy(P->d_boxes, hb.data(), sizeof(DevBox) * nbox, cudaMemcpyHostToDevice);
-    cudaMemcpy(P->d_poffs, poffs.data(), sizeof(int64_t) * (nbox + 1), cudaMemcpyHostToDevice);
+    // in the order of the stream the push runs on; hb and poffs are local
+    e1 = cudaMemcpyAsync(P->d_boxes, hb.data(), sizeof(DevBox) * nbox, cudaMemcpyHostToDevice, s);
+    e2 = cudaMemcpyAsync(P->d_poffs, poffs.data(), sizeof(int64_t) * (nbox + 1),
+                         cudaMemcpyHostToDevice, s);
+    e3 = cudaStreamSynchronize(s);
+    if (e1 || e2 || e3) {
+      c0->err = "pt_push_batch: copy of the box tables failed";
+      return PT_ERR_CUDA;
+    }
     bool ok = cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming) == cudaSuccess;
     for (auto& g : P->groups) {

@@ -461,13 +461,15 @@ static pt_status export_bf16(pt_ctx* c) {
     for (int i = 0; i < 64; ++i) w4s[64 * q + i] = th[OFF_W4 + 64 * q + i] * osc[q];
     b4s[q] = th[OFF_B4 + q] * osc[q];
   }
-  MCK(cudaMemcpy(s->w2b, w2.data(), 4096 * 2, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->w3b, w3.data(), 4096 * 2, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->w1x, w1x.data(), 192 * 4, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->b2, th.data() + OFF_B2, 64 * 4, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->b3, th.data() + OFF_B3, 64 * 4, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->w4s, w4s.data(), 192 * 4, cudaMemcpyHostToDevice));
-  MCK(cudaMemcpy(s->b4s, b4s.data(), 4 * 4, cudaMemcpyHostToDevice));
+  // in the order of the stream that the network runs on (a non-blocking one does
+  // not wait for a plain cudaMemcpy, which may return before its transfer is done)
+  MCK(cudaMemcpyAsync(s->w2b, w2.data(), 4096 * 2, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->w3b, w3.data(), 4096 * 2, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->w1x, w1x.data(), 192 * 4, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->b2, th.data() + OFF_B2, 64 * 4, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->b3, th.data() + OFF_B3, 64 * 4, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->w4s, w4s.data(), 192 * 4, cudaMemcpyHostToDevice, c->stream));
+  MCK(cudaMemcpyAsync(s->b4s, b4s.data(), 4 * 4, cudaMemcpyHostToDevice, c->stream));
   std::memcpy(s->h_w1x, w1x.data(), sizeof s->h_w1x);
   std::memcpy(s->h_b2, th.data() + OFF_B2, sizeof s->h_b2);
   std::memcpy(s->h_b3, th.data() + OFF_B3, sizeof s->h_b3);
@@ -547,7 +549,7 @@ pt_status pt_mlp_set(pt_ctx* c, const float* theta, const float* norm) {
     if (!(norm[51 + q] > 0)) return mfail(c, PT_ERR_ARG, "in_std must be > 0");
   pt_status st = ensure_state(c);
   if (st) return st;
-  MCK(cudaMemcpy(c->mlp->theta, theta, NPAR * 4, cudaMemcpyHostToDevice));
+  MCK(cudaMemcpyAsync(c->mlp->theta, theta, NPAR * 4, cudaMemcpyHostToDevice, c->stream));
   std::memcpy(c->mlp->hnorm, norm, sizeof(float) * NNORM);
   c->mlp->have_theta = true;
   return export_bf16(c);
@@ -609,10 +611,10 @@ pt_status pt_mlp_train(pt_ctx* c, int64_t n, const float* in, const float* tgt, 
     s->hnorm[51 + q] = (float)std::sqrt(std::max(var, 1e-24));
   }
   for (int q = 0; q < 3; ++q) s->hnorm[102 + q] = (float)std::sqrt(std::max(acc[105 + q] / n, 1e-30));
-  MCK(cudaMemcpy(s->norm, s->hnorm, NNORM * 4, cudaMemcpyHostToDevice));
+  MCK(cudaMemcpyAsync(s->norm, s->hnorm, NNORM * 4, cudaMemcpyHostToDevice, c->stream));
   std::vector<float> th;
   init_theta(seed, th);
-  MCK(cudaMemcpy(s->theta, th.data(), NPAR * 4, cudaMemcpyHostToDevice));
+  MCK(cudaMemcpyAsync(s->theta, th.data(), NPAR * 4, cudaMemcpyHostToDevice, c->stream));
   MCK(cudaMemsetAsync(s->grad, 0, NPAR * 4, c->stream));
   MCK(cudaMemsetAsync(s->m, 0, NPAR * 4, c->stream));
   MCK(cudaMemsetAsync(s->v, 0, NPAR * 4, c->stream));
