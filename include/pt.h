@@ -79,12 +79,12 @@ typedef enum { PT_TRACK_PHYSICAL = 0, PT_TRACK_REFERENCE = 1 } pt_track;
 /* Kernel schedule of pt_push.  RESIDENT: one kernel per pt_push chunk keeps
  * every particle in registers for all its stages.  STAGED: one kernel per RK
  * stage over the particle state in element-sorted order (held in library-
- * owned device buffers of about 116 bytes per particle in PT_FP32 mode, 144 in
+ * owned device buffers of about 120 bytes per particle in PT_FP32 mode, 144 in
  * PT_FP64 mode), the stage segments that may cross a face collected in a
  * compacted list and tracked by kernels of their own.  AUTO: STAGED from
  * 2^19 particles on (2^18 with the learned start), RESIDENT below (the list
- * kernels' latency dominates small pushes).  Both run the same arithmetic in the same order per
- * particle. */
+ * kernels' latency dominates small pushes).  Both run the same arithmetic in the
+ * same order per particle. */
 typedef enum { PT_SCHEDULE_AUTO = 0, PT_SCHEDULE_RESIDENT = 1, PT_SCHEDULE_STAGED = 2 } pt_schedule;
 typedef enum {
   PT_DEPOSIT_ATOMIC = 0,     /* FP32 atomics                                   */
@@ -159,7 +159,10 @@ typedef struct {
   int32_t curved_faces; /* intersection with curved faces (Sec. 3.2.4): 0 Newton from
                            the roots of the face's bilinear patch (default; a
                            crossing it misses is found by the walk after the
-                           stage); 1 Bezier clipping of the face's control net   */
+                           stage); 1 Bezier clipping of the face's control net.
+                           PT_FP32 mode: internal and periodic crossings that are
+                           clear in single precision are found by Newton steps in
+                           reference space under either value                     */
   int32_t schedule;     /* pt_schedule: how pt_push maps the stages to kernels
                            (default PT_SCHEDULE_AUTO); results do not depend on it */
   int32_t reserved[2];
@@ -225,6 +228,9 @@ void pt_config_default(pt_config* cfg);
  * builds the per-face tables (face kind by bounding box, Sec. 3.2.4; bilinear
  * coefficients; bounding slabs), the element centres and trilinear start
  * tables.  stream: cudaStream_t used for all later work (NULL = default).
+ * Device memory of the mesh: 1340 bytes per element (connectivity, faces, start)
+ * and its geometry nodes and map coefficients in both precisions, 672, 2484,
+ * 5376 or 11148 bytes per element at ngeo 1, 2, 3 or 4.
  * Returns PT_ERR_ARG for inconsistent connectivity (a neighbour that does not
  * point back, an out-of-range element or face index, a non-periodic face with
  * a shift, a malformed mortar row or one not referenced by exactly one big
@@ -251,8 +257,8 @@ pt_status pt_set_fluid(pt_ctx* ctx, int32_t N, int32_t node_type, const void* U_
  * nsteps x 5 stages interpolate the same U.  A solver that updates U every
  * time step calls pt_push with nsteps = 1 between its own updates (binning
  * and, in the staged schedule, the sorted copy of the particle state are then
- * paid per step); the paper's fully coupled loop, in which the fluid and the
- * particles advance stage by stage together, is not offered.
+ * paid per step); pt_push_stage serves the paper's fully coupled loop, in which
+ * the fluid and the particles advance stage by stage together.
  * Per stage and particle (Sec. 3.2): inverse map x -> xi by Newton, tensor-
  * product interpolation of rho and rho u at xi (Eq. part_interpolation),
  * drag (Eqs. dragforce, dragfactor) plus gravity, the RK update of x and v,
@@ -304,8 +310,8 @@ pt_status pt_push_host(pt_ctx* ctx, const pt_particles* p_host, int32_t nsteps, 
  * PT_DEPOSIT_ATOMIC adds with FP32 atomics (order-dependent rounding);
  * PT_DEPOSIT_SEGMENTED sums each element's particles in index order (bitwise
  * reproducible): it sorts each element's particles by index (O(m^2) for
- * m <= 128 particles in an element, O(m log^2 m) above), computes every particle's source into a
- * library-owned device buffer of 36 bytes per particle (grown on demand,
+ * m <= 128 particles in an element, O(m log^2 m) above), computes every
+ * particle's source into a library-owned device buffer of 36 bytes per particle (grown on demand,
  * released by pt_destroy), then reduces per element.  Other mode bits: PT_ERR_ARG. */
 pt_status pt_deposit(pt_ctx* ctx, const pt_particles* p, int32_t mode, float* S_dev);
 

@@ -1065,14 +1065,19 @@ static cudaEvent_t take_event(pt_ctx* c, int kind = 0) {
 
 // Particles from which PT_SCHEDULE_AUTO takes the staged schedule.  A stage of
 // the staged schedule pays about 60 us for the latency of its list kernels, the
-// resident one nothing; its kernels then run at twice the occupancy.  us per
-// call, resident / staged, 3 steps: NGeo 2, N 5 on 32^3: 1349 / 2492 at 2.5e5
-// particles, 2416 / 3319 at 5e5, 4387 / 4210 at 10^6; NGeo 4, N 6 on 20^3: 2332 /
-// 3124, 4433 / 5055 and 8445 / 7935; FP64, NGeo 2, N 5 on 24^3: 11978 / 14549 and
-// 22708 / 23817.  Where many particles meet walls the resident kernel's warps wait
-// for the FP64 intersections (7e5, NGeo 4, N 6, falling onto a wall: 5.1 ms against
-// 4.6), which puts the line at 2^19.  The learned start's tensor-core kernel exists
-// in the staged schedule only, which is ahead earlier with it.
+// resident one nothing, but where particles meet walls the resident kernel's
+// warps wait for the FP64 intersections, which the staged one compacts (7e5
+// particles, NGeo 4, N 6, falling onto a wall: 5.1 ms against 4.6).  That case
+// sets the line.  Calls in which few particles meet walls pay for it: us per call
+// of 3 steps from a fresh placement, resident / staged: NGeo 2, N 5 on 32^3:
+// 1221 / 2291 at 2.6e5 particles, 2154 / 3186 at 5.3e5, 3697 / 4151 at 10^6; NGeo 3,
+// N 4 on 24^3: 1922 / 2559 at 5.3e5, 3474 / 4060 at 10^6; NGeo 4, N 6 on 20^3: 1878 /
+// 2794 at 2.6e5, 3525 / 4623 at 5.3e5, 6538 / 7574 at 10^6; FP64, NGeo 2, N 5 on 24^3:
+// 22591 / 24410 at 5.3e5, 41099 / 43686 at 10^6.  Further on, once particles have
+// reached the walls, NGeo 2, N 5 on 32^3 takes 2416 / 3319 at 5e5 and 4387 / 4210 at
+// 10^6.  The learned start's tensor-core kernel exists in the staged schedule only;
+// a fresh placement takes 1972 / 3193 at 2.6e5 (NGeo 3, N 5 on 32^3), 3640 / 4530 at
+// 5.3e5.
 static const int64_t kStagedMin = (int64_t)1 << 19, kStagedMinMlp = (int64_t)1 << 18;
 
 static bool use_staged(const pt_ctx* c, int64_t n) {

@@ -6,9 +6,11 @@
 #include "pt_mlp_infer.cuh"
 
 // minimum resident blocks of 128 threads per SM for the push kernel (sets the
-// register budget: 2 -> 255 registers per thread, 3 -> 168, 4 -> 128).  At the
-// 64^3 NGeo=3 workload 2 measured best (FP32: +1-2 % over 3, 3 +8-14 % over 4):
-// spills cost more than the lower occupancy
+// register budget: 2 -> 255 registers per thread, 3 -> 168, 4 -> 128).  Measured at
+// the 64^3 NGeo=3 workload with the element map in Lagrange form, which 2 suited
+// best (FP32: +1-2 % over 3, 3 +8-14 % over 4: spills cost more than the lower
+// occupancy); not measured again with the monomial map, whose kernel still uses
+// 255 registers and spills some 250 bytes
 #ifndef PT_PUSH_MINB
 #define PT_PUSH_MINB 2
 #endif

@@ -7,12 +7,15 @@
 // basis functions, so a point evaluation is G^3 multiply-adds with nothing but
 // the point itself in registers; the Lagrange form spent more on the bases in
 // double-float (~450 instructions) than on anything else.  Two neighbouring
-// powers of xi1 are evaluated per instruction (packed FP32).  On [-1, 1] and
-// degree <= 4 the monomial coefficients are within a factor ~5 of the nodes,
-// so the form costs no accuracy (conversion in FP64, coefficients split in a
-// high and a low FP32 part; largest error of xi over 10^6 points of the 32^3
-// NGeo 3 channel against 64 bits: 3.2e-14 of xi's norm, 3.7e-14 with the Lagrange
-// form in double-float).  The stage kernel went from 7640 to 3200 instructions
+// powers of xi1 are evaluated per instruction (packed FP32).  The
+// conversion can make coefficients larger than the nodes by a factor of 2, 4.5 or
+// 10.7 per direction at degree 2, 3 or 4 (its largest row sum), but the elements of
+// a smooth mesh have coefficients that fall off with the degree, and the form
+// costs no accuracy (conversion in FP64, coefficients split in a high and a low
+// FP32 part): error of xi over 10^6 points of the 32^3 channel against 64 bits at
+// NGeo 1 / 2 / 3 / 4: 6.8e-15 / 9.1e-15 / 3.2e-14 / 2.4e-14 of xi's norm (3.7e-14 at
+// NGeo 3 with the Lagrange form in double-float), at most 6.0e-14 / 8.1e-14 / 1.0e-13 /
+// 1.4e-13.  The stage kernel went from 7640 to 3200 instructions
 // per warp and stage and from 0.45 to 0.255 ns per particle and stage (10^6
 // particles, 32^3, NGeo 2, N 5); point location from 931 to 582 us for 10^6.
 #pragma once
